@@ -418,14 +418,24 @@ pat_status pat_create_grid(const pat_grid_desc* desc, const pat_sampling_desc* s
     }
     if (st == PAT_OK && G->kind == PAT_SAMPLE_POINTS)
         st = upload(G, &G->w.idx, std::vector<int32_t>(sampling->indices, sampling->indices + G->m), "indices");
+    if (st == PAT_OK && G->kind == PAT_SAMPLE_POINTS) {
+        std::vector<int32_t> inv(M, -1);
+        for (int j = 0; j < G->m; j++) inv[sampling->indices[j]] = j;
+        st = upload(G, &G->w.inv, inv, "inverse indices");
+    }
     if (st == PAT_OK && (G->kind == PAT_SAMPLE_HADAMARD01 || G->kind == PAT_SAMPLE_HADAMARDPM)) {
         st = upload(G, &G->w.perm, std::vector<int32_t>(sampling->perm, sampling->perm + M), "perm");
+        const int nt = shd_threads(M), vpt = nt > 0 ? M / nt : 0;
+        std::vector<uint16_t> permt(M);
+        for (int t = 0; t < nt; t++)
+            for (int i = 0; i < vpt; i++) permt[2 * (i / 2 * nt + t) + i % 2] = (uint16_t)sampling->perm[t * vpt + i];
+        if (st == PAT_OK) st = upload(G, &G->w.permt, permt, "perm by thread");
         if (st == PAT_OK)
             st = upload(G, &G->w.rows, std::vector<int32_t>(sampling->rows, sampling->rows + G->m), "rows");
     }
     if (st == PAT_OK) st = build_tables(G);
     if (st == PAT_OK) {
-        e = configure_kernels(g);
+        e = configure_kernels(g, G->kind);
         if (e != cudaSuccess) {
             const std::string where = std::string("configure_kernels (") + configure_failure() + ")";
             st = cuda_fail(e, where.c_str());

@@ -99,7 +99,9 @@ struct Workspace {
     float* rec;                 // real plane series [B][T][M] (sampled kinds); shares memory with
                                 // ms and ph, which are dead whenever it is live
     int32_t* idx;               // POINTS index list
+    int32_t* inv;               // POINTS: the measurement at each plane point, or -1
     int32_t* perm;              // HADAMARD scramble
+    uint16_t* permt;            // the same in the order the transform's threads read it (pat_sample.cu)
     int32_t* rows;              // HADAMARD rows
 };
 
@@ -142,7 +144,8 @@ struct Profiler {
 // Launchers (pat_run.cu, pat_sample.cu).  All return cudaSuccess or the launch error.
 int plane_cluster_size(int nx, int ny);
 const char* configure_failure();  // which attribute the last failed configure_kernels call set
-cudaError_t configure_kernels(const Geom& g);
+cudaError_t configure_kernels(const Geom& g, int kind);
+int shd_threads(int M);  // threads per plane of the Hadamard kernels (0: no kernel for this plane size)
 // workspace layout: bytes of each part (256-byte aligned) for a grid and sampling kind
 struct WsLayout {
     size_t ms[3], ph, rk, rec, total;

@@ -19,7 +19,7 @@
 
 namespace pat {
 
-cudaError_t configure_sampling(const Geom& g);
+cudaError_t configure_sampling(const Geom& g, int kind);
 cudaError_t run_inject_only(const Geom& g, const float* inj, float* p, cudaStream_t st);
 
 #define PAT_TRY(x)                            \
@@ -57,7 +57,7 @@ int plane_cluster_size(int nx, int ny) { return plane_kernels_for(nx, ny).cs; }
 static const char* g_config_what = "";
 const char* configure_failure() { return g_config_what; }
 
-cudaError_t configure_kernels(const Geom& g) {
+cudaError_t configure_kernels(const Geom& g, int kind) {
     PlaneKernels pk = plane_kernels_for(g.nx, g.ny);
     ZKernels zk = z_kernels_for(g.nz);
     if (!pk.rfft || !zk.fwd) {
@@ -85,7 +85,7 @@ cudaError_t configure_kernels(const Geom& g) {
         PAT_CFG(cudaFuncSetAttribute(lk.pass[ax], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lk.smem),
                 "line pass smem");
     }
-    PAT_CFG(configure_sampling(g), "sampling smem");
+    PAT_CFG(configure_sampling(g, kind), "sampling smem");
 #undef PAT_CFG
     g_config_what = "";
     return cudaSuccess;
