@@ -13,7 +13,7 @@
 
 namespace pat {
 cudaError_t conv3_tc(const void* x, int ldx, int cin, const void* w, int cout, void* y, int ldy, int D, int H,
-                     int W, int relu, cudaStream_t st);
+                     int W, int relu, const void* mask, int ldm, cudaStream_t st);
 cudaError_t unet_take_status(int* word, cudaStream_t st);
 void unet_set_copy_fault(int stop_after, int polls);
 int64_t wgrad_tc_scratch(int cin, int cout, int D, int H, int W);
@@ -197,7 +197,7 @@ pat_status pat_unet_conv3(const void* x, int32_t ldx, int32_t cin, const void* w
     if (cout < 16 || cout > 1024 || cout % 16) return bad("pat_unet_conv3: cout must be a multiple of 16 (<= 1024)");
     if (D < 1 || H < 1 || W < 1 || (int64_t)D * H * W > (1LL << 30)) return bad("pat_unet_conv3: bad volume");
     if (!al16(x) || !al16(w) || !al16(y)) return bad("pat_unet_conv3: pointers must be 16-byte aligned");
-    const cudaError_t e = pat::conv3_tc(x, ldx, cin, w, cout, y, ldy, D, H, W, relu, (cudaStream_t)stream);
+    const cudaError_t e = pat::conv3_tc(x, ldx, cin, w, cout, y, ldy, D, H, W, relu, nullptr, 0, (cudaStream_t)stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return pat::set_cuda_error(e, "pat_unet_conv3");

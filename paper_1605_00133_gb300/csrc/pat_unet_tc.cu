@@ -2,19 +2,28 @@
 // (tcgen05): BF16 operands staged by the TMA unit, FP32 accumulators in tensor memory.
 //
 // Implicit GEMM, D[m][n] = sum_k A[m][k] B[n][k] with M = voxels, N = output channels, K = 27 taps x
-// input channels.  A CTA owns one tile of M = 128 voxels, a bx x by x bz box of the volume (x
-// fastest), and BN output channels.  One K step is one tap and CK input channels:
+// input channels, accumulated in the order taps, then channels by 16 (whatever the kernel and its tiles: the
+// result of a layer does not depend on them).  What bounds it, measured:
+//   the MMA, M = 128, K = 16: 46 cycles for N <= 32, 49 at 64, 65 at 128, 129 at 256 -- if the issuing warp
+//     is converged (elect_one);
+//   the TMA unit: one box row (one voxel's channels, up to 64 bytes; 128 bytes in 1.2 cycles) per cycle and
+//     SM, whatever the row's width: so a row of 48 (or 96, ...) channels is fetched as one (two) rows of 64
+//     channels, the missing ones zero-filled, not in 16-channel pieces.
+// conv3_ring_kernel (few channels, large volumes) fetches every line a few times and is bound by its MMAs;
+// conv3_tc_kernel serves every other shape, one shifted box per tap.
+// conv3_tc_kernel: a CTA owns one tile of M = 128 voxels, a bx x by x bz box of the volume (x fastest), and
+// BN output channels.  One K step is one tap and CK input channels:
 //   A: the voxel box shifted by the tap, loaded by a 4D tensor map over (channel, x, y, z); parts of
 //      the box outside the volume come back as zeros, which is the convolution's zero padding;
 //   B: the tap's weights w[t][n0 .. n0+BN)[c0 .. c0+CK), a 3D tensor map over (cin, cout, tap).
 // Both land K-major in shared memory, CK BF16 per row with the swizzle of that row width (32, 64 or
 // 128 bytes), the layout the MMA's shared-memory descriptors read.  Warp roles (192 threads):
-//   warp 0   one thread issues the TMA copies of a NSTAGE-deep ring (full/empty mbarriers);
-//   warp 1   allocates the tensor-memory accumulator (128 lanes x BN FP32 columns) and one thread
-//            issues tcgen05.mma (M = 128, N = BN, K = 16 per instruction), committing each stage's
-//            MMAs to that stage's empty barrier and the last to the done barrier;
+//   warp 0   one thread issues the TMA copies of a ring of stages (full/empty mbarriers);
+//   warp 1   allocates the tensor-memory accumulator (128 lanes x BN FP32 columns) and issues tcgen05.mma
+//            (M = 128, N = BN, K = 16 per instruction), committing each stage's MMAs to that stage's
+//            empty barrier and the last to the done barrier;
 //   warps 2-5 the epilogue: tcgen05.ld of the accumulator rows (warp w reads lanes 32 (w % 4) ..),
-//            optional ReLU, BF16 rounding, one voxel row per thread to global memory.
+//            optional ReLU or mask, BF16 rounding, one voxel row per thread to global memory.
 // Every mbarrier wait is bounded.  A wait that gives up records bit 0 of a device word (read and
 // cleared by pat_unet_device_status), and the CTA stops issuing work, waits (bounded) for the copies
 // it issued, frees its tensor memory and exits; its outputs are then invalid.
@@ -45,6 +54,8 @@ int g_polls = kPolls;
 
 struct ConvTcArgs {
     __nv_bfloat16* y;
+    const __nv_bfloat16* mask;  // NULL: none
+    int ldm;
     int ldy, cin, cout, bn;
     int D, H, W;
     int bx, by, bz;     // voxel box of a tile
@@ -94,11 +105,25 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+// One lane of a converged warp.  The MMA warp runs its loop with all lanes, and only this lane issues: the
+// descriptors are then warp-uniform values.  Issued from inside a one-lane branch an instruction took
+// about 145 cycles (operands moved to uniform registers one by one behind their own arithmetic), three
+// times what the MMA itself takes at N = 48.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+// a descriptor's low word (address field; the descriptors below differ in nothing else within a kernel) and
+// high word are passed separately
+__device__ __forceinline__ uint32_t lo32(uint64_t d) { return (uint32_t)d; }
+__device__ __forceinline__ uint32_t hi32(uint64_t d) { return (uint32_t)(d >> 32); }
+__device__ __forceinline__ void tc_mma(uint32_t tmem_d, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                       uint32_t idesc, uint32_t acc) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc)
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
+        "setp.ne.b32 p, %6, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}" ::"r"(tmem_d),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc)
         : "memory");
 }
 // arrive on `bar` once every tcgen05 operation this thread issued before has completed
@@ -121,6 +146,36 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float* v) {
     for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
 }
 
+// Rounds 16 channels of a voxel to BF16 and stores them.  With a mask (the activation a gradient is taken
+// through) channels where it is not positive are stored as zero.
+__device__ __forceinline__ void conv_store16(const float* v, int relu, const __nv_bfloat16* mask, __nv_bfloat16* out) {
+    uint4 pk[2], mk[2];
+    uint32_t* w32 = reinterpret_cast<uint32_t*>(pk);
+    if (mask) {
+        mk[0] = reinterpret_cast<const uint4*>(mask)[0];
+        mk[1] = reinterpret_cast<const uint4*>(mask)[1];
+    }
+    const __nv_bfloat162* m2 = reinterpret_cast<const __nv_bfloat162*>(mk);
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        float p = v[2 * i], q = v[2 * i + 1];
+        if (relu) {
+            p = fmaxf(p, 0.f);
+            q = fmaxf(q, 0.f);
+        }
+        if (mask) {
+            const float2 mv = __bfloat1622float2(m2[i]);
+            p = mv.x > 0.f ? p : 0.f;
+            q = mv.y > 0.f ? q : 0.f;
+        }
+        const __nv_bfloat162 h = __floats2bfloat162_rn(p, q);
+        w32[i] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    uint4* dst = reinterpret_cast<uint4*>(out);
+    dst[0] = pk[0];
+    dst[1] = pk[1];
+}
+
 template <int CK>
 __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(const __grid_constant__ CUtensorMap tmx,
                                                                 const __grid_constant__ CUtensorMap tmw,
@@ -132,9 +187,10 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(const __grid_cons
     constexpr uint32_t A_BYTES = kBM * RB;     // 4, 8 or 16 KB: a multiple of 1024
     const uint32_t b_bytes = (uint32_t)a.bn * RB;
     const uint32_t stage_bytes = (A_BYTES + b_bytes + 1023) & ~1023u;
-    unsigned long long* full = reinterpret_cast<unsigned long long*>(smem + kNStage * stage_bytes);
-    unsigned long long* empty = full + kNStage;
-    unsigned long long* done = empty + kNStage;
+    constexpr int nstage = kNStage;
+    unsigned long long* full = reinterpret_cast<unsigned long long*>(smem + nstage * stage_bytes);
+    unsigned long long* empty = full + nstage;
+    unsigned long long* done = empty + nstage;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     int* counts = reinterpret_cast<int*>(tmem_slot + 1);  // [0] stages issued, [1] consumed, [2] failed
 
@@ -144,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(const __grid_cons
     const int y0 = ((tile / a.tx) % a.ty) * a.by;
     const int z0 = (tile / (a.tx * a.ty)) * a.bz;
     const int n0 = blockIdx.y * a.bn;
-    const int nc = a.cin / CK;
+    const int nc = (a.cin + CK - 1) / CK;
     const int S = 27 * nc;
     // bytes a stage's two copies deliver: the voxel box (at most 128 rows; rows of the tile beyond it
     // are never stored) and the weight tile
@@ -157,7 +213,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(const __grid_cons
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kNStage; s++) {
+        for (int s = 0; s < nstage; s++) {
             mbar_init(full + s, 1);
             mbar_init(empty + s, 1);
         }
@@ -172,46 +228,71 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(const __grid_cons
 
     if (warp == 0 && lane == 0) {
         // producer
-        int s = 0;
+        int s = 0, st = 0, c0 = 0, t = 0, dx = -1, dy = -1, dz = -1;
+        uint32_t phase = 1;  // a fresh empty barrier's preceding phase counts as complete
         for (; s < S; s++) {
-            const int st = s % kNStage, use = s / kNStage;
             if (a.stop_after >= 0 && s >= a.stop_after) break;  // test hook: nothing more is issued
-            if (use > 0 && !mbar_wait(empty + st, (use - 1) & 1, kPolls)) {
+            if (!mbar_wait(empty + st, phase, kPolls)) {
                 counts[2] = 1;
                 break;
             }
-            const int t = s / nc, c0 = (s - t * nc) * CK;
-            const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
             uint8_t* sa = smem + st * stage_bytes;
             mbar_arrive_expect_tx(full + st, tx_bytes);
             tma_load_4d(sa, &tmx, c0, x0 + dx, y0 + dy, z0 + dz, full + st);
             tma_load_3d(sa + A_BYTES, &tmw, c0, n0, t, full + st);
+            if ((c0 += CK) >= a.cin) {
+                c0 = 0;
+                t++;
+                if (++dx > 1) {
+                    dx = -1;
+                    if (++dy > 1) {
+                        dy = -1;
+                        dz++;
+                    }
+                }
+            }
+            if (++st == nstage) {
+                st = 0;
+                phase ^= 1;
+            }
         }
         counts[0] = s;
-    } else if (warp == 1 && lane == 0) {
-        // MMA issuer
+    } else if (warp == 1) {
+        // MMA issuer (all lanes run the loop, one issues)
+        const bool leader = elect_one();
         const uint32_t idesc = mma_idesc(a.bn);
-        int s = 0;
+        const uint64_t d0 = kmajor_desc(smem_addr(smem), RB);
+        const uint32_t hi = hi32(d0), lo0 = lo32(d0), stage16 = stage_bytes >> 4;
+        int s = 0, st = 0, c0 = 0;
+        uint32_t phase = 0, lo = lo0;
         for (; s < S; s++) {
-            const int st = s % kNStage, use = s / kNStage;
             // the test hook's short limit applies only to the first stage it leaves out
             const int lim = (a.stop_after >= 0 && s >= a.stop_after) ? a.polls : kPolls;
-            if (!mbar_wait(full + st, use & 1, lim)) {
-                counts[2] = 1;
+            if (!__all_sync(0xffffffffu, mbar_wait(full + st, phase, lim))) {
+                if (leader) counts[2] = 1;
                 break;
             }
             tc_fence_after();
-            const uint32_t sa = smem_addr(smem + st * stage_bytes);
+            if (leader) {
 #pragma unroll
-            for (int k = 0; k < CK / 16; k++) {
-                const uint64_t ad = kmajor_desc(sa + 32 * k, RB);
-                const uint64_t bd = kmajor_desc(sa + A_BYTES + 32 * k, RB);
-                tc_mma(tmem, ad, bd, idesc, (s > 0 || k > 0) ? 1u : 0u);
+                for (int k = 0; k < CK / 16; k++)  // 32 bytes along K; channels past cin are zeros, left out
+                    if (c0 + 16 * k < a.cin)
+                        tc_mma(tmem, lo + 2 * k, hi, lo + A_BYTES / 16 + 2 * k, hi, idesc, (s > 0 || k > 0) ? 1u : 0u);
+                tc_commit(empty + st);
             }
-            tc_commit(empty + st);
+            __syncwarp();
+            if ((c0 += CK) >= a.cin) c0 = 0;
+            lo += stage16;
+            if (++st == nstage) {
+                st = 0;
+                phase ^= 1;
+                lo = lo0;
+            }
         }
-        counts[1] = s;
-        tc_commit(done);
+        if (leader) {
+            counts[1] = s;
+            tc_commit(done);
+        }
     } else if (warp >= 2) {
         // epilogue
         const bool ok = mbar_wait(done, 0, kPolls);
@@ -223,27 +304,13 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(const __grid_cons
         const int xx = m % a.bx, yy = (m / a.bx) % a.by, zz = m / (a.bx * a.by);
         const int x = x0 + xx, y = y0 + yy, z = z0 + zz;
         const bool valid = ok && m < a.bx * a.by * a.bz && x < a.W && y < a.H && z < a.D;
-        __nv_bfloat16* out = a.y + ((size_t)((size_t)z * a.H + y) * a.W + x) * a.ldy + n0;
+        const size_t vox = ((size_t)z * a.H + y) * a.W + x;  // used only where valid
+        __nv_bfloat16* out = a.y + vox * a.ldy + n0;
+        const __nv_bfloat16* mask = a.mask + vox * a.ldm + n0;
         for (int c = 0; c < a.bn; c += 16) {
             float v[16];
             tc_ld16(trow + (uint32_t)c, v);  // every thread of the warp takes part
-            if (valid) {
-                uint4 pk[2];
-                uint32_t* w32 = reinterpret_cast<uint32_t*>(pk);
-#pragma unroll
-                for (int i = 0; i < 8; i++) {
-                    float p = v[2 * i], q = v[2 * i + 1];
-                    if (a.relu) {
-                        p = fmaxf(p, 0.f);
-                        q = fmaxf(q, 0.f);
-                    }
-                    const __nv_bfloat162 h = __floats2bfloat162_rn(p, q);
-                    w32[i] = *reinterpret_cast<const uint32_t*>(&h);
-                }
-                uint4* dst = reinterpret_cast<uint4*>(out + c);
-                dst[0] = pk[0];
-                dst[1] = pk[1];
-            }
+            if (valid) conv_store16(v, a.relu, a.mask ? mask + c : nullptr, out + c);
         }
     }
     tc_fence_before();
@@ -252,7 +319,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(const __grid_cons
         if (threadIdx.x == 0) {
             atomicOr(&g_unet_err, 1);
             // copies issued but never consumed may still be in flight: let them land (bounded)
-            for (int s = counts[1]; s < counts[0]; s++) mbar_wait(full + s % kNStage, (s / kNStage) & 1, kPolls);
+            for (int s = counts[1]; s < counts[0]; s++) mbar_wait(full + s % nstage, (s / nstage) & 1, kPolls);
             mbar_wait(done, 0, kPolls);
         }
         __syncthreads();
@@ -265,26 +332,258 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(const __grid_cons
 }
 
 // ---------------------------------------------------------------------------------------------
-// Weight gradient: dW[t][co][ci] = sum_v dY[v][co] X[v + off_t][ci], all 27 taps in one GEMM with
-// M = (tap, input channel) rows m = t cin + ci (M tiles along grid.x, so that the CTAs reading one
-// voxel chunk run together and find its input in L2), N = output channels and K = voxels, split over
-// chunks of voxel blocks (grid.y) with a fixed-order sum afterwards.  A K block is a box of 64 voxels.  Both
-// operands arrive channel-contiguous, i.e. MN-major: a swizzle atom is 8 voxel rows x WA channels of
-// one tap (A) or 8 voxel rows x WB output channels (B), WA, WB in {16, 32, 64}; the M tile's 128 rows
-// are 128 / WA atoms side by side (one TMA box each: the tap's shifted voxel box, zero outside the
-// volume), the N tile's cout columns cout / WB atoms.  In a descriptor the leading byte offset steps
-// from one atom to the next along M or N, the stride byte offset from one 8-row group of voxels to
-// the next.
+// The same convolution for few channels on large volumes (lines up to 128 voxels, weights that fit shared
+// memory): a persistent kernel.  A CTA keeps its weights in shared memory and walks along z through a
+// column of one M tile (by lines of W voxels), holding a ring of input planes of by + 2 lines; steps
+// (column, z) are numbered column by column and each CTA takes an equal contiguous range.  A tap's operand
+// is 128 rows of a plane from another start: dz planes, dy lines and dx voxels on.
+//   Lines over 64 voxels (by = 1): a plane's lines are W + 2 voxels (x = -1 .. W), in parts of 16 channels
+//     (32-byte rows), up to four; the operand starts dy (W + 2) + dx rows on.  The 32-byte swizzle is applied
+//     to shared-memory address bits by the TMA unit and the tensor core alike, so any row may be the first.
+//   Shorter lines (16 or 32 channels): every plane is held three times, shifted by dx, its lines bx voxels (W
+//     rounded up to 8), so that operands start at multiples of 8 rows and by lines fill the 128 rows.
+// Per tile the MMAs, 27 per 16 channels, are what is left: 27 x 46 = 1242 cycles at 16 channels, beside 390
+// rows (cycles) of the TMA unit; the epilogue works on a ring of accumulators, two groups of four warps
+// taking alternate tiles.  64x128x128 voxels: 16 -> 16 channels 137 -> 50 us, 48 -> 16 371 -> 114 us,
+// 16 -> 48 379 -> 54 us (one box per tap, and MMAs issued from one lane, before).
+// Other shapes use the kernel above: longer lines, more channels (weights and planes do not fit, and its K
+// steps are bound less by the TMA unit), and volumes of less than four tiles an SM (the weights would be
+// fetched for too little work).
+// ---------------------------------------------------------------------------------------------
+
+constexpr int kRingThreads = 320;  // producer, MMA issuer, 2 x 4 epilogue warps
+constexpr int kMaxPlanes = 8, kMaxAcc = 8;
+
+struct ConvRingArgs {
+    __nv_bfloat16* y;
+    const __nv_bfloat16* mask;  // NULL: none
+    int ldm;
+    int ldy, cin, bn;
+    int D, H, W;
+    int pitch, by, lines;     // rows from line to line; a tile is by lines, a plane of the ring by + 2
+    int ncopies;              // copies of a plane shifted by dx (1: the lines have a halo), from x = -1
+    int steps_per_cta, steps; // (column, z) steps
+    int relu;
+    int nplanes, nacc, acc_cols;
+    uint32_t box_bytes;       // one part of one copy of a plane
+    uint32_t dxstep;          // from tap dx to dx + 1, in 16-byte units: a copy or a row
+};
+
+template <int CK, int NP>  // NP parts of CK input channels
+__global__ void __launch_bounds__(kRingThreads, 1)
+    conv3_ring_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmw, ConvRingArgs a) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    __shared__ unsigned long long pfull[kMaxPlanes], pempty[kMaxPlanes], tfull[kMaxAcc], tempty[kMaxAcc], wfull, done;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int failed;
+    constexpr uint32_t RB = CK * 2;  // bytes per operand row = swizzle width
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t plane_bytes = a.ncopies * NP * a.box_bytes;
+    uint8_t* planes = smem;
+    uint8_t* wts = smem + a.nplanes * plane_bytes;
+    const int n0 = blockIdx.y * a.bn;
+    const int u0 = blockIdx.x * a.steps_per_cta, u1 = min(a.steps, u0 + a.steps_per_cta);
+
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_slot)),
+                     "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < a.nplanes; i++) {
+            mbar_init(pfull + i, 1);
+            mbar_init(pempty + i, 1);
+        }
+        for (int i = 0; i < a.nacc; i++) {
+            mbar_init(tfull + i, 1);
+            mbar_init(tempty + i, 4);  // one arrival per epilogue warp
+        }
+        mbar_init(&wfull, 1);
+        mbar_init(&done, 1);
+        mbar_fence_init();
+        failed = 0;
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+
+    if (warp == 0 && lane == 0) {
+        // producer: the weights, then the planes z-1 .. z+1 of every step in order, each once per run of z
+        mbar_arrive_expect_tx(&wfull, 27u * NP * a.bn * RB);
+        for (int q = 0; q < NP; q++) tma_load_3d(wts + q * 27 * a.bn * RB, &tmw, q * CK, n0, 0, &wfull);
+        const uint32_t tx_bytes = (uint32_t)(a.ncopies * NP * a.pitch * a.lines) * RB;
+        int p = 0, slot = 0;
+        uint32_t phase = 1;  // a fresh empty barrier's preceding phase counts as complete
+        bool ok = true;
+        for (int u = u0; u < u1 && ok;) {
+            const int col = u / a.D, z0 = u - col * a.D, n = min(u1 - u, a.D - z0);
+            for (int z = z0 - 1; z <= z0 + n; z++, p++) {
+                if (!mbar_wait(pempty + slot, phase, kPolls)) {
+                    ok = false;
+                    break;
+                }
+                uint8_t* d = planes + slot * plane_bytes;
+                mbar_arrive_expect_tx(pfull + slot, tx_bytes);
+                for (int k = 0; k < a.ncopies; k++)
+                    for (int q = 0; q < NP; q++, d += a.box_bytes)
+                        tma_load_4d(d, &tmx, q * CK, k - 1, col * a.by - 1, z, pfull + slot);
+                if (++slot == a.nplanes) {
+                    slot = 0;
+                    phase ^= 1;
+                }
+            }
+            u += n;
+        }
+        if (!ok) atomicOr(&failed, 1);
+        // let every copy issued land before this CTA's shared memory can go to another (bounded)
+        mbar_wait(&wfull, 0, kPolls);
+        for (int k = max(0, p - a.nplanes); k < p; k++) mbar_wait(pfull + k % a.nplanes, (k / a.nplanes) & 1, kPolls);
+    } else if (warp == 1) {
+        // MMA issuer (all lanes run the loop, one issues)
+        const bool leader = elect_one();
+        const uint32_t idesc = mma_idesc(a.bn);
+        const uint64_t da = kmajor_desc(smem_addr(planes), RB), db = kmajor_desc(smem_addr(wts), RB);
+        const uint32_t hi = hi32(da);
+        // address steps in 16-byte units: a plane, a part, dx, a line, one tap's weights, a part's
+        const uint32_t pstep = plane_bytes >> 4, qstep = a.box_bytes >> 4, dxstep = a.dxstep;
+        const uint32_t lstep = a.pitch * (RB / 16), wstep = a.bn * (RB / 16), wqstep = 27 * wstep;
+        bool ok = mbar_wait(&wfull, 0, kPolls);
+        int slot = 0, acc = 0;      // ring slot of the next plane to wait for, accumulator
+        uint32_t pphase = 0, acc_phase = 1;
+        int first = 0;              // ring slot of plane z - 1 of the current step
+        for (int u = u0; u < u1 && ok;) {
+            const int col = u / a.D, z0 = u - col * a.D, n = min(u1 - u, a.D - z0);
+            for (int i = 0; i < n; i++) {
+                for (int k = (i == 0) ? 3 : 1; k > 0 && ok; k--) {
+                    ok = mbar_wait(pfull + slot, pphase, kPolls);
+                    if (++slot == a.nplanes) {
+                        slot = 0;
+                        pphase ^= 1;
+                    }
+                }
+                ok = ok && mbar_wait(tempty + acc, acc_phase, kPolls);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t td = tmem + acc * a.acc_cols;
+                const bool last = i + 1 == n;
+                if (leader) {
+#pragma unroll
+                    for (int dz = 0; dz < 3; dz++) {
+                        int sl = first + dz;
+                        if (sl >= a.nplanes) sl -= a.nplanes;
+#pragma unroll
+                        for (int r = 0; r < 9; r++) {
+                            const uint32_t x = lo32(da) + sl * pstep + (r % 3) * dxstep + (r / 3) * lstep;
+                            const uint32_t w = lo32(db) + (9 * dz + r) * wstep;
+#pragma unroll
+                            for (int q = 0; q < NP; q++) {
+                                tc_mma(td, x + q * qstep, hi, w + q * wqstep, hi, idesc, (dz + r + q) ? 1u : 0u);
+                                if (CK == 32) tc_mma(td, x + 2, hi, w + 2, hi, idesc, 1);
+                            }
+                        }
+                        // plane z - 1 is done with here; after the last step of a run all three are
+                        if (dz == 0 || last) tc_commit(pempty + sl);
+                    }
+                    tc_commit(tfull + acc);
+                }
+                __syncwarp();
+                first += last ? 3 : 1;
+                if (first >= a.nplanes) first -= a.nplanes;
+                if (++acc == a.nacc) {
+                    acc = 0;
+                    acc_phase ^= 1;
+                }
+            }
+            u += n;
+        }
+        if (leader) {
+            if (!ok) atomicOr(&failed, 1);
+            tc_commit(&done);
+        }
+        __syncwarp();
+        mbar_wait(&done, 0, kPolls);  // every MMA has finished before the tensor memory is freed
+    } else if (warp >= 2) {
+        const int grp = (warp - 2) >> 2, m = 32 * (warp & 3) + lane;
+        const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+        const int xx = m % a.pitch, yy = m / a.pitch;
+        int acc = 0, turn = 0, col = u0 / a.D, z = u0 - col * a.D;
+        uint32_t acc_phase = 0;
+        bool ok = true;
+        for (int u = u0; u < u1 && ok; u++) {
+            if (turn == grp) {
+                ok = __all_sync(0xffffffffu, mbar_wait(tfull + acc, acc_phase, kPolls));
+                tc_fence_after();
+                const int y = col * a.by + yy;
+                const bool valid = ok && yy < a.by && xx < a.W && y < a.H;
+                const size_t vox = ((size_t)z * a.H + y) * a.W + xx;  // used only where valid
+                __nv_bfloat16* out = a.y + vox * a.ldy + n0;
+                const __nv_bfloat16* mask = a.mask + vox * a.ldm + n0;
+                const uint32_t td = trow + acc * a.acc_cols;
+                for (int c = 0; c < a.bn; c += 16) {
+                    float v[16];
+                    tc_ld16(td + c, v);
+                    if (c + 16 >= a.bn) {  // the accumulator is in registers
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0)
+                            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(tempty + acc)) : "memory");
+                    }
+                    if (valid) conv_store16(v, a.relu, a.mask ? mask + c : nullptr, out + c);
+                }
+            }
+            turn ^= 1;
+            if (++z == a.D) {
+                z = 0;
+                col++;
+            }
+            if (++acc == a.nacc) {
+                acc = 0;
+                acc_phase ^= 1;
+            }
+        }
+        if (!ok) atomicOr(&failed, 1);
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (failed && threadIdx.x == 0) atomicOr(&g_unet_err, 1);
+    if (warp == 1) {
+        __syncwarp();
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Weight gradient: dW[t][co][ci] = sum_v dY[v][co] X[v + off_t][ci] = sum_u dY[u - dx][co] X[u + (dz,dy)][ci],
+// all 27 taps in one GEMM: M = (dz, dy) x input channels, N = dx x output channels, K = voxels, split
+// over chunks of voxel blocks with a fixed-order sum afterwards.  With the tap's shift shared between
+// the operands a block is fetched as 9 shifted boxes of X and 3 of dY, where 27 shifted boxes of X (and dY
+// once per M tile) took 27 box rows a voxel of the TMA unit's one per cycle (see the file comment).
+// A K block is a box of 64 voxels.  Both operands arrive channel-contiguous, i.e. MN-major: a
+// swizzle atom is 8 voxel rows x WA channels of one (dz, dy) (A) or 8 voxel rows x WB output channels of
+// one dx (B), WA, WB in {16, 32, 64}, zero-filled past cin; an M tile's 128 rows are 128 / WA atoms side by
+// side (one TMA box each, zero outside the volume), the N columns 3 BN / WB atoms.  In a descriptor the
+// leading byte offset steps from one atom to the next along M or N, the stride byte offset from one
+// 8-row group of voxels to the next.  A CTA accumulates several M tiles (as many as fit the tensor
+// memory with their N columns and three stages of shared memory), so one fetch of a block serves them all.  The boxes of a stage are issued
+// by the lanes of the producer warp together, each its own (coordinates and destinations are fixed
+// per lane but for the block).
 // ---------------------------------------------------------------------------------------------
 
 constexpr int kKB = 64;  // voxels per K block
 
 struct WgradArgs {
-    float* partial;     // [chunk][mtiles * 128][cout]
-    int cin, cout, wa, wb;
+    float* partial;     // [chunk][mtiles * 128][3 cout]
+    int cin, cout, bn, wa, wb;
+    int mtiles, mt;     // M tiles in all, per CTA
     int D, H, W;
     int bx, by, bz, tx, ty, nkb;   // voxel box of a K block, blocks along x and y, blocks in all
     int kb_per_cta;
+    int nstage;
     uint32_t tmem_cols;
 };
 
@@ -305,29 +604,35 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_tc_kernel(const __grid_cons
                                                                WgradArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const uint32_t ra = 2u * a.wa, rb = 2u * a.wb;      // row bytes = swizzle widths
+    const uint32_t ra = 2u * a.wa, rb = 2u * a.wb;       // row bytes = swizzle widths
     const uint32_t atom_a = kKB * ra, atom_b = kKB * rb; // one atom column over the K block
-    const uint32_t a_bytes = kBM * kKB * 2;              // 16 KB
-    const uint32_t b_bytes = (uint32_t)a.cout * kKB * 2;
+    constexpr uint32_t tile_bytes = kBM * kKB * 2;       // one M tile: 16 KB
+    const uint32_t a_bytes = a.mt * tile_bytes;
+    const int N = 3 * a.bn;
+    const int ncols = (N + 31) & ~31;                    // tensor-memory columns of an M tile
+    const uint32_t b_bytes = (uint32_t)N * kKB * 2;
     const uint32_t stage_bytes = (a_bytes + b_bytes + 1023) & ~1023u;
-    unsigned long long* full = reinterpret_cast<unsigned long long*>(smem + kNStage * stage_bytes);
-    unsigned long long* empty = full + kNStage;
-    unsigned long long* done = empty + kNStage;
+    const int nstage = a.nstage;
+    unsigned long long* full = reinterpret_cast<unsigned long long*>(smem + nstage * stage_bytes);
+    unsigned long long* empty = full + nstage;
+    unsigned long long* done = empty + nstage;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     int* counts = reinterpret_cast<int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int mtile = blockIdx.x;  // M tiles fastest: the CTAs of one voxel chunk run together
+    const int mgroups = (a.mtiles + a.mt - 1) / a.mt;
+    const int mtile0 = (blockIdx.x % mgroups) * a.mt, ng = blockIdx.x / mgroups;  // M tiles, output channels
+    const int mt = min(a.mt, a.mtiles - mtile0);
     const int chunk = blockIdx.y;
     const int kb0 = chunk * a.kb_per_cta;
     const int nkb = min(a.kb_per_cta, a.nkb - kb0);
-    const int natoms_a = kBM / a.wa;                 // atoms (tap, channel block) of this M tile
-    const int cblocks = a.cin / a.wa;
-    const int atom0 = mtile * natoms_a;
-    const int atoms_total = 27 * cblocks;
-    const int natoms_live = min(natoms_a, atoms_total - atom0);
-    const int nb_atoms = a.cout / a.wb;
-    const uint32_t tx_bytes = (uint32_t)natoms_live * atom_a + b_bytes;
+    const int per_tile = kBM / a.wa;                 // atoms (dz dy, channel block) of an M tile
+    const int cblocks = (a.cin + a.wa - 1) / a.wa;
+    const int atom0 = mtile0 * per_tile;
+    const int na = min(mt * per_tile, 9 * cblocks - atom0);  // atoms of this CTA that exist
+    const int nbb = a.bn / a.wb;                     // atoms per dx
+    const int nbox = na + 3 * nbb;
+    const uint32_t tx_bytes = (uint32_t)na * atom_a + b_bytes;
 
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
@@ -336,7 +641,7 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_tc_kernel(const __grid_cons
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kNStage; s++) {
+        for (int s = 0; s < nstage; s++) {
             mbar_init(full + s, 1);
             mbar_init(empty + s, 1);
         }
@@ -349,51 +654,90 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_tc_kernel(const __grid_cons
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp == 0 && lane == 0) {
-        int s = 0;
+    if (warp == 0) {
+        // this lane's box of every stage (nbox <= 32, checked by the launch)
+        const CUtensorMap* map = &tmx;
+        int c0 = 0, dx = 0, dy = 0, dz = 0;
+        uint32_t dst = 0;
+        if (lane < na) {
+            const int atom = atom0 + lane, row = atom / cblocks;
+            c0 = (atom - row * cblocks) * a.wa;
+            dy = row % 3 - 1;
+            dz = row / 3 - 1;
+            dst = lane * atom_a;
+        } else {
+            const int e = lane - na, d = e / nbb;
+            map = &tmd;
+            c0 = ng * a.bn + (e - d * nbb) * a.wb;
+            dx = 1 - d;  // tap dx = d - 1 reads dY at u - dx
+            dst = a_bytes + e * atom_b;
+        }
+        int tx = kb0 % a.tx, ty = (kb0 / a.tx) % a.ty, tz = kb0 / (a.tx * a.ty);
+        int s = 0, st = 0;
+        uint32_t phase = 1;  // a fresh empty barrier's preceding phase counts as complete
         for (; s < nkb; s++) {
-            const int st = s % kNStage, use = s / kNStage;
-            if (use > 0 && !mbar_wait(empty + st, (use - 1) & 1, kPolls)) {
-                counts[2] = 1;
+            if (!__all_sync(0xffffffffu, mbar_wait(empty + st, phase, kPolls))) {
+                if (lane == 0) counts[2] = 1;
                 break;
             }
-            const int kb = kb0 + s;
-            const int x0 = (kb % a.tx) * a.bx, y0 = ((kb / a.tx) % a.ty) * a.by, z0 = (kb / (a.tx * a.ty)) * a.bz;
-            uint8_t* sa = smem + st * stage_bytes;
-            mbar_arrive_expect_tx(full + st, tx_bytes);
-            for (int j = 0; j < natoms_live; j++) {
-                const int atom = atom0 + j, t = atom / cblocks, c0 = (atom - t * cblocks) * a.wa;
-                const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
-                tma_load_4d(sa + j * atom_a, &tmx, c0, x0 + dx, y0 + dy, z0 + dz, full + st);
+            if (lane == 0) mbar_arrive_expect_tx(full + st, tx_bytes);
+            __syncwarp();
+            if (lane < nbox)
+                tma_load_4d(smem + st * stage_bytes + dst, map, c0, tx * a.bx + dx, ty * a.by + dy, tz * a.bz + dz,
+                            full + st);
+            if (++tx == a.tx) {
+                tx = 0;
+                if (++ty == a.ty) {
+                    ty = 0;
+                    tz++;
+                }
             }
-            for (int j = 0; j < nb_atoms; j++)
-                tma_load_4d(sa + a_bytes + j * atom_b, &tmd, j * a.wb, x0, y0, z0, full + st);
+            if (++st == nstage) {
+                st = 0;
+                phase ^= 1;
+            }
         }
-        counts[0] = s;
-    } else if (warp == 1 && lane == 0) {
-        // A and B MN-major (bits 15, 16), FP32 accumulator, BF16 operands, M = 128, N = cout
+        if (lane == 0) counts[0] = s;
+    } else if (warp == 1) {
+        // A and B MN-major (bits 15, 16), FP32 accumulator, BF16 operands, M = 128; all lanes run the loop,
+        // one issues
+        const bool leader = elect_one();
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
-                               ((uint32_t)(a.cout >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-        int s = 0;
+                               ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
+        const uint64_t ad = mnmajor_desc(smem_addr(smem), ra, atom_a), bd = mnmajor_desc(smem_addr(smem) + a_bytes, rb, atom_b);
+        const uint32_t ahi = hi32(ad), bhi = hi32(bd), stage16 = stage_bytes >> 4, tile16 = tile_bytes >> 4;
+        int s = 0, st = 0;
+        uint32_t phase = 0, off = 0;
         for (; s < nkb; s++) {
-            const int st = s % kNStage, use = s / kNStage;
-            if (!mbar_wait(full + st, use & 1, kPolls)) {
-                counts[2] = 1;
+            if (!__all_sync(0xffffffffu, mbar_wait(full + st, phase, kPolls))) {
+                if (leader) counts[2] = 1;
                 break;
             }
             tc_fence_after();
-            const uint32_t sa = smem_addr(smem + st * stage_bytes);
-#pragma unroll
-            for (int k = 0; k < kKB / 16; k++) {
+            if (leader) {
                 // 16 voxel rows = two 8-row groups: the start moves by 16 rows of each operand
-                const uint64_t ad = mnmajor_desc(sa + 16 * ra * k, ra, atom_a);
-                const uint64_t bd = mnmajor_desc(sa + a_bytes + 16 * rb * k, rb, atom_b);
-                tc_mma(tmem, ad, bd, idesc, (s > 0 || k > 0) ? 1u : 0u);
+                const uint32_t blo = lo32(bd) + off;
+                uint32_t alo = lo32(ad) + off, td = tmem;
+                const uint32_t on = s > 0 ? 1u : 0u;
+                for (int t = 0; t < mt; t++, alo += tile16, td += ncols) {
+#pragma unroll
+                    for (int k = 0; k < kKB / 16; k++)
+                        tc_mma(td, alo + k * ra, ahi, blo + k * rb, bhi, idesc, k ? 1u : on);
+                }
+                tc_commit(empty + st);
             }
-            tc_commit(empty + st);
+            __syncwarp();
+            off += stage16;
+            if (++st == nstage) {
+                st = 0;
+                phase ^= 1;
+                off = 0;
+            }
         }
-        counts[1] = s;
-        tc_commit(done);
+        if (leader) {
+            counts[1] = s;
+            tc_commit(done);
+        }
     } else if (warp >= 2) {
         const bool ok = mbar_wait(done, 0, kPolls);
         if (!ok) counts[2] = 1;
@@ -401,17 +745,15 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_tc_kernel(const __grid_cons
         tc_fence_after();
         const int m = 32 * (warp & 3) + lane;
         const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
-        float* out = a.partial + ((size_t)chunk * gridDim.x * kBM + (size_t)mtile * kBM + m) * a.cout;
-        for (int c = 0; c < a.cout; c += 16) {
-            float v[16];
-            tc_ld16(trow + (uint32_t)c, v);
-            if (nkb <= 0) {
+        for (int t = 0; t < mt; t++) {
+            float* out = a.partial + (((size_t)chunk * a.mtiles + mtile0 + t) * kBM + m) * (3 * a.cout) + ng * N;
+            for (int c = 0; c < N; c += 16) {
+                float v[16];
+                tc_ld16(trow + (uint32_t)(t * ncols + c), v);
+                float4* dst = reinterpret_cast<float4*>(out + c);
 #pragma unroll
-                for (int i = 0; i < 16; i++) v[i] = 0.f;
+                for (int i = 0; i < 4; i++) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
             }
-            float4* dst = reinterpret_cast<float4*>(out + c);
-#pragma unroll
-            for (int i = 0; i < 4; i++) dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
         }
     }
     tc_fence_before();
@@ -419,7 +761,7 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_tc_kernel(const __grid_cons
     if (counts[2]) {
         if (threadIdx.x == 0) {
             atomicOr(&g_unet_err, 1);
-            for (int s = counts[1]; s < counts[0]; s++) mbar_wait(full + s % kNStage, (s / kNStage) & 1, kPolls);
+            for (int s = counts[1]; s < counts[0]; s++) mbar_wait(full + s % nstage, (s / nstage) & 1, kPolls);
             mbar_wait(done, 0, kPolls);
         }
         __syncthreads();
@@ -431,18 +773,38 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_tc_kernel(const __grid_cons
     }
 }
 
-// dw[t][co][ci] = sum over chunks c (in order) of partial[c][t cin + ci][co]
-__global__ void wgrad_sum_kernel(const float* __restrict__ partial, int nchunk, int rows, int cin, int cout,
-                                 float* __restrict__ dw) {
-    const long long n = 27LL * cin * cout;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int ci = (int)(i % cin);
-        const long long r = i / cin;
-        const int co = (int)(r % cout), t = (int)(r / cout);
-        const size_t row = (size_t)t * cin + ci;
-        float s = 0.f;
-        for (int c = 0; c < nchunk; c++) s += partial[((size_t)c * rows + row) * cout + co];
-        dw[i] = s;
+// dw[3 row + d][co][ci] = sum over chunks of partial[chunk][(row, channel block, ci)][(co / bn, d, co % bn)].
+// A CTA takes 32 product columns of R rows; S threads share the chunks of each sum (a serial loop of one
+// thread over 152 chunks is a chain of memory latencies), their parts added in a fixed order.  R = 8
+// consecutive input channels are written together (32 bytes), worth it when there are few chunks and so
+// many outputs.  27 x 16 x 16 outputs of 152 chunks (R = 1, S = 16): 28 -> 8 us; 27 x 192 x 64 of 20 (R = 8,
+// S = 2): 20 -> 13 us.
+template <int R, int S>
+__global__ void __launch_bounds__(32 * R * S) wgrad_sum_kernel(const float* __restrict__ partial, int nchunk, int rows,
+                                                               int cin, int cout, int bn, int wa,
+                                                               float* __restrict__ dw) {
+    __shared__ float sh[S][R][33];
+    const int lane = threadIdx.x & 31, r = (threadIdx.x >> 5) % R, sl = threadIdx.x / (32 * R);
+    const int ncol = 3 * cout, cblocks = (cin + wa - 1) / wa;
+    const int m0 = blockIdx.y * R, col = blockIdx.x * 32 + lane;
+    float s = 0.f;
+    if (col < ncol) {
+        const float* p = partial + (size_t)(m0 + r) * ncol + col;
+        const size_t cs = (size_t)rows * ncol;
+#pragma unroll 10
+        for (int c = sl; c < nchunk; c += S) s += p[c * cs];
+    }
+    sh[sl][r][lane] = s;
+    __syncthreads();
+    if (threadIdx.x < 32 * R) {
+        const int ro = threadIdx.x % R, co0 = threadIdx.x / R, c = blockIdx.x * 32 + co0, m = m0 + ro;
+        const int atom = m / wa, row = atom / cblocks, ci = (atom - row * cblocks) * wa + m % wa;
+        if (c < ncol && ci < cin) {  // (ci >= cin: a zero-filled channel)
+            float t = sh[0][ro][co0];
+            for (int k = 1; k < S; k++) t += sh[k][ro][co0];
+            const int g = c / (3 * bn), q = c - g * 3 * bn, d = q / bn, co = g * bn + q - d * bn;
+            dw[((size_t)(3 * row + d) * cout + co) * cin + ci] = t;
+        }
     }
 }
 
@@ -482,20 +844,116 @@ cudaError_t launch_ck(const CUtensorMap& mx, const CUtensorMap& mw, const ConvTc
 
 }  // namespace
 
+// a K-major operand map: channels c of a (channel, x, y, z) or (cin, cout, tap) tensor in boxes of ck of them
+static CUresult kmajor_map(CUtensorMap* m, int rank, const void* p, const cuuint64_t* dims, const cuuint64_t* strides,
+                           const cuuint32_t* box) {
+    const cuuint32_t es[4] = {1, 1, 1, 1};
+    const CUtensorMapSwizzle swz = box[0] == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+                                   : box[0] == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                                  : CU_TENSOR_MAP_SWIZZLE_32B;
+    return encoder()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(p), dims, strides, box, es,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+}
+
+// Geometry of conv3_ring_kernel; ctas = 0 where the other kernel serves the shape.
+struct RingGeom {
+    ConvRingArgs a;
+    int ctas, groups, ck;  // ck: channels of a part
+    size_t smem;
+};
+static RingGeom ring_geom(int cin, int cout, int D, int H, int W) {
+    RingGeom g = {};
+    ConvRingArgs& a = g.a;
+    const bool halo = W > 64;
+    if (W > kBM || cin > (halo ? 64 : 32)) return g;
+    a.cin = cin;
+    a.D = D;
+    a.H = H;
+    a.W = W;
+    g.ck = halo ? 16 : cin;
+    a.pitch = halo ? W + 2 : (W + 7) & ~7;
+    a.by = halo ? 1 : std::min(H, kBM / a.pitch);
+    a.lines = a.by + 2;
+    a.ncopies = halo ? 1 : 3;
+    a.box_bytes = (uint32_t)(a.lines * a.pitch * g.ck * 2 + 1023) & ~1023u;
+    a.dxstep = halo ? (uint32_t)g.ck / 8 : a.box_bytes >> 4;
+    const size_t plane = (size_t)a.ncopies * (cin / g.ck) * a.box_bytes;
+    // the largest share of the output channels whose weights fit beside three planes; an operand reads up to
+    // 128 rows past its box: 8 KB of pad follow the weights
+    constexpr size_t kRoom = 227 * 1024 - 1024 - 1024 - 8192;
+    for (int n = 1; n <= 8 && !a.bn; n++)
+        if (cout % (16 * n) == 0 && cout / n <= 128 && (size_t)27 * (cout / n) * cin * 2 + 3 * plane <= kRoom) {
+            g.groups = n;
+            a.bn = cout / n;
+        }
+    if (!a.bn) return g;
+    const size_t wbytes = (size_t)27 * a.bn * cin * 2;
+    const int ytiles = (H + a.by - 1) / a.by, sms = 152 / g.groups;
+    a.steps = ytiles * D;
+    if ((long long)ytiles * D < 4LL * sms) return g;
+    a.steps_per_cta = (a.steps + sms - 1) / sms;
+    a.acc_cols = (a.bn + 31) & ~31;
+    a.nacc = std::min(kMaxAcc, 512 / a.acc_cols);
+    a.nplanes = (int)std::min<size_t>(kMaxPlanes, (kRoom - wbytes) / plane);
+    g.ctas = (a.steps + a.steps_per_cta - 1) / a.steps_per_cta;
+    g.smem = 1024 + a.nplanes * plane + wbytes + 8192;
+    // one CTA per SM (it holds all of the tensor memory): more than half of the shared memory
+    g.smem = std::max(g.smem, (size_t)(120 * 1024));
+    return g;
+}
+
+static cudaError_t launch_ring(RingGeom& g, const void* x, int ldx, const void* w, int cout, cudaStream_t st) {
+    const ConvRingArgs& a = g.a;
+    alignas(64) CUtensorMap mx, mw;
+    const cuuint64_t xd[4] = {(cuuint64_t)a.cin, (cuuint64_t)a.W, (cuuint64_t)a.H, (cuuint64_t)a.D};
+    const cuuint64_t xs[3] = {(cuuint64_t)ldx * 2, (cuuint64_t)ldx * 2 * a.W, (cuuint64_t)ldx * 2 * a.W * a.H};
+    const cuuint32_t xb[4] = {(cuuint32_t)g.ck, (cuuint32_t)a.pitch, (cuuint32_t)a.lines, 1};
+    const cuuint64_t wd[3] = {(cuuint64_t)a.cin, (cuuint64_t)cout, 27};
+    const cuuint64_t ws[2] = {(cuuint64_t)a.cin * 2, (cuuint64_t)a.cin * 2 * cout};
+    const cuuint32_t wb[3] = {(cuuint32_t)g.ck, (cuuint32_t)a.bn, 27};
+    if (kmajor_map(&mx, 4, x, xd, xs, xb) != CUDA_SUCCESS || kmajor_map(&mw, 3, w, wd, ws, wb) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    const int np = a.cin / g.ck;
+    const auto kernel = g.ck == 32 ? conv3_ring_kernel<32, 1>
+                        : np == 1  ? conv3_ring_kernel<16, 1>
+                        : np == 2  ? conv3_ring_kernel<16, 2>
+                        : np == 3  ? conv3_ring_kernel<16, 3>
+                                   : conv3_ring_kernel<16, 4>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+    if (e != cudaSuccess) return e;
+    kernel<<<dim3((unsigned)g.ctas, (unsigned)g.groups), kRingThreads, g.smem, st>>>(mx, mw, a);
+    return cudaGetLastError();
+}
+
 // y[v][n] = act(sum_t sum_c x[v + off_t][c] w[t][n][c]) on the tensor cores (see the file comment).
 // Channel counts multiples of 16, strides multiples of 16 elements, pointers 16-byte aligned (checked
 // by the caller).
 cudaError_t conv3_tc(const void* x, int ldx, int cin, const void* w, int cout, void* y, int ldy, int D, int H,
-                     int W, int relu, cudaStream_t st) {
+                     int W, int relu, const void* mask, int ldm, cudaStream_t st) {
     EncodeTiled enc = encoder();
     if (!enc) return cudaErrorNotSupported;
-    const int ck = (cin % 64 == 0) ? 64 : (cin % 32 == 0) ? 32 : 16;
+    RingGeom ring = ring_geom(cin, cout, D, H, W);
+    if (ring.ctas > 0 && g_stop_after < 0) {
+        ring.a.y = reinterpret_cast<__nv_bfloat16*>(y);
+        ring.a.ldy = ldy;
+        ring.a.relu = relu;
+        ring.a.mask = reinterpret_cast<const __nv_bfloat16*>(mask);
+        ring.a.ldm = ldm;
+        return launch_ring(ring, x, ldx, w, cout, st);
+    }
+    // channels per operand row: one row where cin fits in it (16, 32), else pieces of 64, the last one
+    // zero-filled past cin
+    const int ck = cin == 16 ? 16 : cin == 32 ? 32 : 64;
     ConvTcArgs a = {};
     a.y = reinterpret_cast<__nv_bfloat16*>(y);
     a.ldy = ldy;
     a.cin = cin;
     a.cout = cout;
-    a.bn = (cout % 128 == 0) ? 128 : (cout % 64 == 0) ? 64 : (cout % 32 == 0) ? 32 : 16;
+    // output channels per CTA: the largest divisor up to 128, so that a tile's voxels are fetched for as many
+    // channels as fit; but where the tiles alone do not give every SM a CTA, fewer
+    for (int n = 1; !a.bn; n++)
+        if (cout % (16 * n) == 0 && cout / n <= 128) a.bn = cout / n;
     a.D = D;
     a.H = H;
     a.W = W;
@@ -508,32 +966,21 @@ cudaError_t conv3_tc(const void* x, int ldx, int cin, const void* w, int cout, v
     const long long tiles = (long long)a.tx * a.ty * tz;
     if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
     a.relu = relu;
-    a.tmem_cols = a.bn < 32 ? 32 : a.bn;
+    a.mask = reinterpret_cast<const __nv_bfloat16*>(mask);
+    a.ldm = ldm;
+    while (a.bn > 16 && tiles * (cout / a.bn) < 152 && cout % (a.bn / 2) == 0 && (a.bn / 2) % 16 == 0) a.bn /= 2;
+    a.tmem_cols = a.bn <= 32 ? 32 : a.bn <= 64 ? 64 : 128;
     a.stop_after = g_stop_after;
     a.polls = g_polls;
-    const CUtensorMapSwizzle swz =
-        ck == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : ck == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B;
     alignas(64) CUtensorMap mx, mw;
-    {
-        const cuuint64_t dims[4] = {(cuuint64_t)cin, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)D};
-        const cuuint64_t strides[3] = {(cuuint64_t)ldx * 2, (cuuint64_t)ldx * 2 * W, (cuuint64_t)ldx * 2 * W * H};
-        const cuuint32_t box[4] = {(cuuint32_t)ck, (cuuint32_t)a.bx, (cuuint32_t)a.by, (cuuint32_t)a.bz};
-        const cuuint32_t es[4] = {1, 1, 1, 1};
-        if (enc(&mx, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(x), dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
-    }
-    {
-        const cuuint64_t dims[3] = {(cuuint64_t)cin, (cuuint64_t)cout, 27};
-        const cuuint64_t strides[2] = {(cuuint64_t)cin * 2, (cuuint64_t)cin * 2 * cout};
-        const cuuint32_t box[3] = {(cuuint32_t)ck, (cuuint32_t)a.bn, 1};
-        const cuuint32_t es[3] = {1, 1, 1};
-        if (enc(&mw, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(w), dims, strides, box, es,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-            return cudaErrorInvalidValue;
-    }
+    const cuuint64_t xd[4] = {(cuuint64_t)cin, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)D};
+    const cuuint64_t xs[3] = {(cuuint64_t)ldx * 2, (cuuint64_t)ldx * 2 * W, (cuuint64_t)ldx * 2 * W * H};
+    const cuuint32_t xb[4] = {(cuuint32_t)ck, (cuuint32_t)a.bx, (cuuint32_t)a.by, (cuuint32_t)a.bz};
+    const cuuint64_t wd[3] = {(cuuint64_t)cin, (cuuint64_t)cout, 27};
+    const cuuint64_t ws[2] = {(cuuint64_t)cin * 2, (cuuint64_t)cin * 2 * cout};
+    const cuuint32_t wb[3] = {(cuuint32_t)ck, (cuuint32_t)a.bn, 1};
+    if (kmajor_map(&mx, 4, x, xd, xs, xb) != CUDA_SUCCESS || kmajor_map(&mw, 3, w, wd, ws, wb) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
     if (ck == 64) return launch_ck<64>(mx, mw, a, (unsigned)tiles, st);
     if (ck == 32) return launch_ck<32>(mx, mw, a, (unsigned)tiles, st);
     return launch_ck<16>(mx, mw, a, (unsigned)tiles, st);
@@ -541,13 +988,40 @@ cudaError_t conv3_tc(const void* x, int ldx, int cin, const void* w, int cout, v
 
 // Geometry of the weight-gradient GEMM (shared by the scratch-size query and the launch).
 struct WgradGeom {
-    int wa, wb, bx, by, bz, tx, ty, nkb, mtiles, kb_per_cta, nchunk;
+    int wa, wb, bn, bx, by, bz, tx, ty, nkb, mtiles, mt, mgroups, ngroups, nstage, kb_per_cta, nchunk;
+    uint32_t tmem_cols;
+    size_t smem;
 };
 
 static WgradGeom wgrad_geom(int cin, int cout, int D, int H, int W) {
     WgradGeom g;
-    g.wa = (cin % 64 == 0) ? 64 : (cin % 32 == 0) ? 32 : 16;
-    g.wb = (cout % 64 == 0) ? 64 : (cout % 32 == 0) ? 32 : 16;
+    g.wa = cin == 16 ? 16 : cin == 32 ? 32 : 64;
+    g.bn = 16;  // output channels per CTA, N = 3 bn <= 256
+    for (int b : {80, 64, 48, 32})
+        if (cout % b == 0) {
+            g.bn = b;
+            break;
+        }
+    g.wb = (g.bn % 64 == 0) ? 64 : (g.bn % 32 == 0) ? 32 : 16;
+    g.ngroups = cout / g.bn;
+    const int atoms = 9 * ((cin + g.wa - 1) / g.wa), N = 3 * g.bn;
+    g.mtiles = (atoms * g.wa + kBM - 1) / kBM;
+    // M tiles per CTA: as many as the 512 tensor-memory columns and three stages of shared memory hold,
+    // spread evenly over the groups
+    auto stage_bytes = [&](int mt) { return (size_t)((mt * kBM + N) * kKB * 2 + 1023) & ~(size_t)1023; };
+    constexpr size_t kSmem = 227 * 1024 - 1024 - 256;
+    const int ncols = (N + 31) & ~31;
+    int mt = std::min(g.mtiles, 512 / ncols);
+    while (mt > 1 && 3 * stage_bytes(mt) > kSmem) mt--;
+    g.mgroups = (g.mtiles + mt - 1) / mt;
+    g.mt = (g.mtiles + g.mgroups - 1) / g.mgroups;
+    g.mgroups = (g.mtiles + g.mt - 1) / g.mt;
+    g.nstage = (int)std::min<size_t>(6, kSmem / stage_bytes(g.mt));
+    g.smem = 1024 + g.nstage * stage_bytes(g.mt) + (2 * g.nstage + 1) * 8 + 4 + 16;
+    const int cols = g.mt * ncols;
+    g.tmem_cols = cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512;
+    // no more CTAs on an SM than tensor memory serves at once (228 KB per SM, 1 KB reserved per CTA)
+    g.smem = std::max(g.smem, (size_t)(233472 / (512 / g.tmem_cols + 1) + 1));
     // a K block is exactly kKB voxels (the MMA reads all its rows): powers of two, the box reaching
     // past the volume where a side is shorter (those voxels read as zeros)
     auto pow2_at_least = [](int v) {
@@ -562,11 +1036,11 @@ static WgradGeom wgrad_geom(int cin, int cout, int D, int H, int W) {
     g.ty = (H + g.by - 1) / g.by;
     const long long tz = (D + g.bz - 1) / g.bz;
     g.nkb = (int)((long long)g.tx * g.ty * tz);
-    g.mtiles = (27 * cin + kBM - 1) / kBM;
-    // about four CTAs per SM over all M tiles, at least 8 K blocks each
-    const long long want = 4LL * 152;
-    long long per = ((long long)g.nkb * g.mtiles + want - 1) / want;
-    if (per < 8) per = 8;
+    // one round of CTAs over the SMs (as many as fit each), at least 4 K blocks each
+    const int per_sm = std::max(1, std::min((int)(512 / g.tmem_cols), (int)(233472 / (g.smem + 1024))));
+    const long long want = std::max(1LL, 152LL * per_sm / (g.mgroups * g.ngroups));
+    long long per = (g.nkb + want - 1) / want;
+    if (per < 4) per = 4;
     g.kb_per_cta = (int)per;
     g.nchunk = (g.nkb + g.kb_per_cta - 1) / g.kb_per_cta;
     return g;
@@ -574,7 +1048,7 @@ static WgradGeom wgrad_geom(int cin, int cout, int D, int H, int W) {
 
 int64_t wgrad_tc_scratch(int cin, int cout, int D, int H, int W) {
     const WgradGeom g = wgrad_geom(cin, cout, D, H, W);
-    return (int64_t)g.nchunk * g.mtiles * kBM * cout;
+    return (int64_t)g.nchunk * g.mtiles * kBM * 3 * cout;
 }
 
 // dw[t][co][ci] = sum_v dy[v][co] x[v + off_t][ci] on the tensor cores; partial: wgrad_tc_scratch
@@ -584,6 +1058,7 @@ cudaError_t wgrad_tc(const void* x, int ldx, int cin, const void* dy, int ldy, i
     EncodeTiled enc = encoder();
     if (!enc) return cudaErrorNotSupported;
     const WgradGeom g = wgrad_geom(cin, cout, D, H, W);
+    if (g.mt * (kBM / g.wa) + 3 * (g.bn / g.wb) > 32) return cudaErrorInvalidValue;  // boxes a stage: one a lane
     const CUtensorMapSwizzle sa = g.wa == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : g.wa == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
                                                                                       : CU_TENSOR_MAP_SWIZZLE_32B;
     const CUtensorMapSwizzle sb = g.wb == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : g.wb == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
@@ -612,8 +1087,11 @@ cudaError_t wgrad_tc(const void* x, int ldx, int cin, const void* dy, int ldy, i
     a.partial = partial;
     a.cin = cin;
     a.cout = cout;
+    a.bn = g.bn;
     a.wa = g.wa;
     a.wb = g.wb;
+    a.mtiles = g.mtiles;
+    a.mt = g.mt;
     a.D = D;
     a.H = H;
     a.W = W;
@@ -624,20 +1102,20 @@ cudaError_t wgrad_tc(const void* x, int ldx, int cin, const void* dy, int ldy, i
     a.ty = g.ty;
     a.nkb = g.nkb;
     a.kb_per_cta = g.kb_per_cta;
-    a.tmem_cols = cout <= 32 ? 32 : cout <= 64 ? 64 : cout <= 128 ? 128 : 256;
-    const uint32_t stage = (kBM * kKB * 2 + cout * kKB * 2 + 1023) & ~1023u;
-    size_t smem = 1024 + kNStage * (size_t)stage + (2 * kNStage + 1) * 8 + 4 + 16;
-    const size_t max_ctas = 512 / a.tmem_cols;
-    const size_t floor_smem = 233472 / (max_ctas + 1) + 1;
-    if (smem < floor_smem) smem = floor_smem;
-    cudaError_t e = cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    a.nstage = g.nstage;
+    a.tmem_cols = g.tmem_cols;
+    cudaError_t e = cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
     if (e != cudaSuccess) return e;
-    wgrad_tc_kernel<<<dim3((unsigned)g.mtiles, (unsigned)g.nchunk), kThreads, smem, st>>>(mx, md, a);
+    wgrad_tc_kernel<<<dim3((unsigned)(g.mgroups * g.ngroups), (unsigned)g.nchunk), kThreads, g.smem, st>>>(mx, md, a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const long long n = 27LL * cin * cout;
-    const int blocks = (int)((n + 255) / 256 < 152 * 8 ? (n + 255) / 256 : 152 * 8);
-    wgrad_sum_kernel<<<blocks, 256, 0, st>>>(partial, g.nchunk, g.mtiles * kBM, cin, cout, dw);
+    const int rows = g.mtiles * kBM, used = 9 * ((cin + g.wa - 1) / g.wa) * g.wa;
+    const unsigned gx = (unsigned)((3 * cout + 31) / 32);
+    if (g.nchunk > 48)
+        wgrad_sum_kernel<1, 16><<<dim3(gx, (unsigned)used), 512, 0, st>>>(partial, g.nchunk, rows, cin, cout, g.bn, g.wa, dw);
+    else
+        wgrad_sum_kernel<8, 2><<<dim3(gx, (unsigned)(used / 8)), 512, 0, st>>>(partial, g.nchunk, rows, cin, cout, g.bn,
+                                                                             g.wa, dw);
     return cudaGetLastError();
 }
 
