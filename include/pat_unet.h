@@ -35,6 +35,13 @@ extern "C" {
 pat_status pat_unet_conv3(const void* x, int32_t ldx, int32_t cin, const void* w, int32_t cout, void* y,
                           int32_t ldy, int32_t D, int32_t H, int32_t W, int32_t relu, void* cuda_stream);
 
+/* The convolution of a gradient taken through the ReLU in front of the layer: y = conv3(x, w) with zeros
+ * where act <= 0, act [V][lda] the activation (cout channels, lda a multiple of 16).  The same values as
+ * pat_unet_conv3 without relu followed by pat_unet_relu_bwd, in one pass. */
+pat_status pat_unet_conv3_masked(const void* x, int32_t ldx, int32_t cin, const void* w, int32_t cout, void* y,
+                                 int32_t ldy, int32_t D, int32_t H, int32_t W, const void* act, int32_t lda,
+                                 void* cuda_stream);
+
 /* Synchronises cuda_stream, then reads and clears the device word in which the tensor-core
  * convolutions record a bounded wait that gave up: PAT_OK, or PAT_ERR_TIMEOUT (the outputs of the
  * convolutions since the last check are invalid). */
@@ -75,12 +82,20 @@ pat_status pat_unet_pool(const void* x, int32_t ldx, int32_t C, int32_t D, int32
 pat_status pat_unet_pool_bwd_add(const void* dy, int32_t ldd, int32_t C, int32_t D, int32_t H, int32_t W,
                                  void* dx, int32_t ldx, void* cuda_stream);
 
+/* The same followed by pat_unet_relu_bwd(dx, act), in one pass. */
+pat_status pat_unet_pool_bwd_add_masked(const void* dy, int32_t ldd, int32_t C, int32_t D, int32_t H, int32_t W,
+                                        void* dx, int32_t ldx, const void* act, int32_t lda, void* cuda_stream);
+
 /* Nearest-neighbour 2x upsampling: x [D][H][W][.] -> y [2D][2H][2W][.]; backward sums the 8
  * children: dx[parent] = sum dy[child] (dims of x given). */
 pat_status pat_unet_up(const void* x, int32_t ldx, int32_t C, int32_t D, int32_t H, int32_t W, void* y,
                        int32_t ldy, void* cuda_stream);
 pat_status pat_unet_up_bwd(const void* dy, int32_t ldd, int32_t C, int32_t D, int32_t H, int32_t W,
                            void* dx, int32_t ldx, void* cuda_stream);
+
+/* pat_unet_up_bwd followed by pat_unet_relu_bwd(dx, act), in one pass. */
+pat_status pat_unet_up_bwd_masked(const void* dy, int32_t ldd, int32_t C, int32_t D, int32_t H, int32_t W, void* dx,
+                                  int32_t ldx, const void* act, int32_t lda, void* cuda_stream);
 
 /* Network input: x16 [V][16] bf16 with channel 0 = s * xin[v] (FP32) and channels 1..15 zero. */
 pat_status pat_unet_input(const float* xin, float s, int64_t V, void* x16, void* cuda_stream);
@@ -96,6 +111,11 @@ int64_t pat_unet_head_scratch(int64_t V);
 pat_status pat_unet_head_bwd(const void* h, const float* head, const float* out, const float* target,
                              int64_t V, void* dh, float* ghead, double* loss, double* partial,
                              void* cuda_stream);
+
+/* The same with dh taken through the ReLU whose output is h (zero where h <= 0). */
+pat_status pat_unet_head_bwd_masked(const void* h, const float* head, const float* out, const float* target,
+                                    int64_t V, void* dh, float* ghead, double* loss, double* partial,
+                                    void* cuda_stream);
 
 /* Adam step on n FP32 parameters: m = b1 m + (1-b1) g, v = b2 v + (1-b2) g^2,
  * p -= lr * (m / (1 - b1^step)) / (sqrt(v / (1 - b2^step)) + eps). */

@@ -24,7 +24,8 @@ EXPORTS = ["pat_create_grid", "pat_destroy_grid", "pat_grid_info", "pat_workspac
 UNET_EXPORTS = ["pat_unet_conv3", "pat_unet_wgrad_scratch", "pat_unet_conv3_wgrad", "pat_unet_cast_weights",
                 "pat_unet_relu_bwd", "pat_unet_pool", "pat_unet_pool_bwd_add", "pat_unet_up", "pat_unet_up_bwd",
                 "pat_unet_input", "pat_unet_head", "pat_unet_head_scratch", "pat_unet_head_bwd", "pat_unet_adam",
-                "pat_unet_device_status", "pat_unet_debug_copy_fault"]
+                "pat_unet_device_status", "pat_unet_debug_copy_fault", "pat_unet_conv3_masked",
+                "pat_unet_pool_bwd_add_masked", "pat_unet_up_bwd_masked", "pat_unet_head_bwd_masked"]
 
 
 class PatError(RuntimeError):
@@ -131,6 +132,10 @@ def load() -> ctypes.CDLL:
         L.pat_unet_head_scratch.argtypes = [i64]
         L.pat_unet_head_scratch.restype = i64
         L.pat_unet_head_bwd.argtypes = [vp, vp, vp, vp, i64, vp, vp, vp, vp, vp]
+        L.pat_unet_conv3_masked.argtypes = [vp, i32, i32, vp, i32, vp, i32, i32, i32, i32, vp, i32, vp]
+        L.pat_unet_pool_bwd_add_masked.argtypes = [vp, i32, i32, i32, i32, i32, vp, i32, vp, i32, vp]
+        L.pat_unet_up_bwd_masked.argtypes = [vp, i32, i32, i32, i32, i32, vp, i32, vp, i32, vp]
+        L.pat_unet_head_bwd_masked.argtypes = [vp, vp, vp, vp, i64, vp, vp, vp, vp, vp]
         L.pat_unet_adam.argtypes = [vp, vp, vp, vp, i64, f32, f32, f32, f32, i32, vp]
         L.pat_unet_device_status.argtypes = [vp]
         L.pat_unet_debug_copy_fault.argtypes = [i32, i32]

@@ -120,14 +120,16 @@ class WarmStartUNet:
         D, H, W = self.dims[lev]
         _lib.check(self.L.pat_unet_conv3(x, ldx, cin, w, cout, y, ldy, D, H, W, int(relu), self._st()))
 
+    def _conv_masked(self, x, ldx, cin, w, cout, y, ldy, lev, act, lda):
+        """data gradient through a layer and the ReLU in front of it, whose output is act"""
+        D, H, W = self.dims[lev]
+        _lib.check(self.L.pat_unet_conv3_masked(x, ldx, cin, w, cout, y, ldy, D, H, W, act, lda, self._st()))
+
     def _wgrad(self, name, x, ldx, dy, ldy):
         cin, cout, lev = LAYERS[name]
         D, H, W = self.dims[lev]
         _lib.check(self.L.pat_unet_conv3_wgrad(x, ldx, cin, dy, ldy, cout, D, H, W, self.wscratch.data_ptr(),
                                                self._g32(name), self._st()))
-
-    def _relu_bwd(self, g, ldg, y, ldy, C, lev):
-        _lib.check(self.L.pat_unet_relu_bwd(g, ldg, y, ldy, C, self.V[lev], self._st()))
 
     # ------------------------------------------------------------------ forward
     def forward(self, xin: torch.Tensor) -> torch.Tensor:
@@ -169,62 +171,51 @@ class WarmStartUNet:
         d0, d1, d2, d3 = self.dims
         wt = {k: v.data_ptr() for k, v in self.wt.items()}
         target = target.reshape(-1).contiguous()
-        _lib.check(L.pat_unet_head_bwd(p(self.h), self._w32("head"), self.out.data_ptr(), target.data_ptr(),
-                                       self.V[0], p(self.dh), self._g32("head"), self.loss_buf.data_ptr(),
-                                       self.hscratch.data_ptr(), st))
+        _lib.check(L.pat_unet_head_bwd_masked(p(self.h), self._w32("head"), self.out.data_ptr(),
+                                              target.data_ptr(), self.V[0], p(self.dh), self._g32("head"),
+                                              self.loss_buf.data_ptr(), self.hscratch.data_ptr(), st))
         # level 1, decoder
-        self._relu_bwd(p(self.dh), 16, p(self.h), 16, 16, 0)
         self._wgrad("d1b", p(self.t1b), 16, p(self.dh), 16)
-        self._conv(p(self.dh), 16, 16, wt["d1b"], 16, p(self.dt1b), 16, 0, False)
-        self._relu_bwd(p(self.dt1b), 16, p(self.t1b), 16, 16, 0)
+        self._conv_masked(p(self.dh), 16, 16, wt["d1b"], 16, p(self.dt1b), 16, 0, p(self.t1b), 16)
         self._wgrad("d1a", p(self.c1), 48, p(self.dt1b), 16)
         self._conv(p(self.dt1b), 16, 16, wt["d1a"], 48, p(self.dc1), 48, 0, False)
-        _lib.check(L.pat_unet_up_bwd(p(self.dc1), 48, 32, *d1, p(self.du2), 32, st))
+        _lib.check(L.pat_unet_up_bwd_masked(p(self.dc1), 48, 32, *d1, p(self.du2), 32, p(self.u2), 32, st))
         # level 2, decoder
-        self._relu_bwd(p(self.du2), 32, p(self.u2), 32, 32, 1)
         self._wgrad("d2b", p(self.t2b), 32, p(self.du2), 32)
-        self._conv(p(self.du2), 32, 32, wt["d2b"], 32, p(self.dt2b), 32, 1, False)
-        self._relu_bwd(p(self.dt2b), 32, p(self.t2b), 32, 32, 1)
+        self._conv_masked(p(self.du2), 32, 32, wt["d2b"], 32, p(self.dt2b), 32, 1, p(self.t2b), 32)
         self._wgrad("d2a", p(self.c2), 96, p(self.dt2b), 32)
         self._conv(p(self.dt2b), 32, 32, wt["d2a"], 96, p(self.dc2), 96, 1, False)
-        _lib.check(L.pat_unet_up_bwd(p(self.dc2), 96, 64, *d2, p(self.du3), 64, st))
+        _lib.check(L.pat_unet_up_bwd_masked(p(self.dc2), 96, 64, *d2, p(self.du3), 64, p(self.u3), 64, st))
         # level 3, decoder
-        self._relu_bwd(p(self.du3), 64, p(self.u3), 64, 64, 2)
         self._wgrad("d3b", p(self.t3b), 64, p(self.du3), 64)
-        self._conv(p(self.du3), 64, 64, wt["d3b"], 64, p(self.dt3b), 64, 2, False)
-        self._relu_bwd(p(self.dt3b), 64, p(self.t3b), 64, 64, 2)
+        self._conv_masked(p(self.du3), 64, 64, wt["d3b"], 64, p(self.dt3b), 64, 2, p(self.t3b), 64)
         self._wgrad("d3a", p(self.c3), 192, p(self.dt3b), 64)
         self._conv(p(self.dt3b), 64, 64, wt["d3a"], 192, p(self.dc3), 192, 2, False)
-        _lib.check(L.pat_unet_up_bwd(p(self.dc3), 192, 128, *d3, p(self.du4), 128, st))
+        _lib.check(L.pat_unet_up_bwd_masked(p(self.dc3), 192, 128, *d3, p(self.du4), 128, p(self.u4), 128, st))
         # level 4
-        self._relu_bwd(p(self.du4), 128, p(self.u4), 128, 128, 3)
         self._wgrad("e4b", p(self.t4), 128, p(self.du4), 128)
-        self._conv(p(self.du4), 128, 128, wt["e4b"], 128, p(self.dt4), 128, 3, False)
-        self._relu_bwd(p(self.dt4), 128, p(self.t4), 128, 128, 3)
+        self._conv_masked(p(self.du4), 128, 128, wt["e4b"], 128, p(self.dt4), 128, 3, p(self.t4), 128)
         self._wgrad("e4a", p(self.p3), 64, p(self.dt4), 128)
         self._conv(p(self.dt4), 128, 128, wt["e4a"], 64, p(self.dp3), 64, 3, False)
         # level 3, encoder (the skip's gradient from the concatenation plus the pooled path)
-        _lib.check(L.pat_unet_pool_bwd_add(p(self.dp3), 64, 64, *d2, p(self.dc3, 128), 192, st))
-        self._relu_bwd(p(self.dc3, 128), 192, p(self.c3, 128), 192, 64, 2)
+        _lib.check(L.pat_unet_pool_bwd_add_masked(p(self.dp3), 64, 64, *d2, p(self.dc3, 128), 192,
+                                                  p(self.c3, 128), 192, st))
         self._wgrad("e3b", p(self.t3), 64, p(self.dc3, 128), 192)
-        self._conv(p(self.dc3, 128), 192, 64, wt["e3b"], 64, p(self.dt3), 64, 2, False)
-        self._relu_bwd(p(self.dt3), 64, p(self.t3), 64, 64, 2)
+        self._conv_masked(p(self.dc3, 128), 192, 64, wt["e3b"], 64, p(self.dt3), 64, 2, p(self.t3), 64)
         self._wgrad("e3a", p(self.p2), 32, p(self.dt3), 64)
         self._conv(p(self.dt3), 64, 64, wt["e3a"], 32, p(self.dp2), 32, 2, False)
         # level 2, encoder
-        _lib.check(L.pat_unet_pool_bwd_add(p(self.dp2), 32, 32, *d1, p(self.dc2, 64), 96, st))
-        self._relu_bwd(p(self.dc2, 64), 96, p(self.c2, 64), 96, 32, 1)
+        _lib.check(L.pat_unet_pool_bwd_add_masked(p(self.dp2), 32, 32, *d1, p(self.dc2, 64), 96,
+                                                  p(self.c2, 64), 96, st))
         self._wgrad("e2b", p(self.t2), 32, p(self.dc2, 64), 96)
-        self._conv(p(self.dc2, 64), 96, 32, wt["e2b"], 32, p(self.dt2), 32, 1, False)
-        self._relu_bwd(p(self.dt2), 32, p(self.t2), 32, 32, 1)
+        self._conv_masked(p(self.dc2, 64), 96, 32, wt["e2b"], 32, p(self.dt2), 32, 1, p(self.t2), 32)
         self._wgrad("e2a", p(self.p1), 16, p(self.dt2), 32)
         self._conv(p(self.dt2), 32, 32, wt["e2a"], 16, p(self.dp1), 16, 1, False)
         # level 1, encoder
-        _lib.check(L.pat_unet_pool_bwd_add(p(self.dp1), 16, 16, *d0, p(self.dc1, 32), 48, st))
-        self._relu_bwd(p(self.dc1, 32), 48, p(self.c1, 32), 48, 16, 0)
+        _lib.check(L.pat_unet_pool_bwd_add_masked(p(self.dp1), 16, 16, *d0, p(self.dc1, 32), 48,
+                                                  p(self.c1, 32), 48, st))
         self._wgrad("e1b", p(self.t1), 16, p(self.dc1, 32), 48)
-        self._conv(p(self.dc1, 32), 48, 16, wt["e1b"], 16, p(self.dt1), 16, 0, False)
-        self._relu_bwd(p(self.dt1), 16, p(self.t1), 16, 16, 0)
+        self._conv_masked(p(self.dc1, 32), 48, 16, wt["e1b"], 16, p(self.dt1), 16, 0, p(self.t1), 16)
         self._wgrad("e1a", p(self.x16), 16, p(self.dt1), 16)
         return self.loss_buf
 
