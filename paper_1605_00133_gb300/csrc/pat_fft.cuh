@@ -247,6 +247,30 @@ __device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, unsign
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)) : "memory");
 }
+// The same copies, and a store, marked evict-first in the L2 (EF): data read and written once per pass that will
+// have left the L2 by its next use anyway, so that it does not displace what will not.
+__device__ __forceinline__ unsigned long long evict_first() {
+    unsigned long long p;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+template <bool EF>
+__device__ __forceinline__ void bulk_copy_g2s_once(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
+    if (EF)
+        asm volatile(
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
+            ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)), "l"(evict_first()) : "memory");
+    else
+        bulk_copy_g2s(dst, src, bytes, bar);
+}
+template <bool EF>
+__device__ __forceinline__ void store_once(float2* p, float2 v, unsigned long long policy) {
+    if (EF)
+        asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1, %2}, %3;" ::"l"(p), "f"(v.x), "f"(v.y), "l"(policy)
+                     : "memory");
+    else
+        *p = v;
+}
 // Wait for phase `parity` of an mbarrier to complete: each poll suspends the thread for at most about
 // a microsecond, and after `polls` polls (about a second for 1 << 20) the wait gives up and returns
 // false; the caller records the failure and does not use what the copy should have delivered, so no
@@ -274,6 +298,15 @@ __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
+}
+template <bool EF>
+__device__ __forceinline__ void cp_async16_once(void* smem, const void* gmem, unsigned long long policy) {
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    if (EF)
+        asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(s), "l"(gmem), "l"(policy)
+                     : "memory");
+    else
+        cp_async16(smem, gmem);
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>

@@ -106,7 +106,8 @@ typedef void (*LineKernel)(LineArgs);
 // where a pair's row group and half are xr = r/2, xh = r%2, or with pnew xh = bit 1 of r and xr
 // the other bits of r
 struct LineKernels {
-    LineKernel pass[3] = {nullptr, nullptr, nullptr};  // by axis (z, y, x) for this line length
+    // by [states streamed past the L2][axis (z, y, x)] for this line length
+    LineKernel pass[2][3] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
     size_t smem = 0;
     int tc = 0;  // lines per CTA (one tile of the state layout)
     int nt = 0;  // threads per CTA

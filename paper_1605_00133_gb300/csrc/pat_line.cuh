@@ -46,6 +46,12 @@
 // plus a compile-time offset.  The twiddles of the two transform halves come from per-thread tables
 // (twi, twf: entry k of thread r at k * (row stride) + r) for the same reason.
 //
+// STREAM: the states are loaded and stored evict-first in the L2, for grids whose loop does not fit it.  Their 48
+// bytes per voxel and step then cross DRAM in any case, and left alone they also displace the two spectra and
+// the kappa tables, which are read three times a step.  128x256x256: 672 -> 598 MB of DRAM traffic a step, a
+// forward and adjoint over 200 steps 66.7 -> 62.7 ms; 64x128x128 with four volumes a call 7.86 -> 7.33 ms over
+// 100 steps.  Where the loop fits (one volume of 64x128x128) the plain accesses are 0.7 % faster.
+//
 // Spectrum access per axis (3D half spectrum [kz][kx][ky], kx <= nx/2):
 //   z lines (kx, ky): column access, stride nxh*ny
 //   y lines (kz, kx): each line is a contiguous row; the CTA's TC rows are one contiguous block,
@@ -125,7 +131,7 @@ __device__ __forceinline__ float2 wr(int k) {
     return make_float2(w16c(k * (16 / R)), DIR * w16s(k * (16 / R)));
 }
 
-template <int L, int AX>
+template <int L, int AX, bool STREAM>
 struct LineCtx {
     using S = LS<L>;
     static constexpr int A = S::A, B = S::B, TC = S::TC, XN = S::XN;
@@ -399,6 +405,7 @@ struct LineCtx {
     // (old values from the prefetched tile pf)
     __device__ __forceinline__ void update(float2* __restrict__ st, const float* const* c, bool no_old,
                                            const float2* pf, float2* x) const {
+        const unsigned long long pol = STREAM ? evict_first() : 0;
         if (xact) {
 #pragma unroll
             for (int q = 0; q < XN; q++) {
@@ -413,7 +420,7 @@ struct LineCtx {
                     nv.x = fmaf(d, o.x, nv.x);
                     nv.y = fmaf(d, o.y, nv.y);
                 }
-                st[sidx(q)] = nv;
+                store_once<STREAM>(st + sidx(q), nv, pol);
                 x[q] = c[2] ? cscale(nv, rd(c[2] + jc)) : nv;
             }
         }
@@ -441,12 +448,12 @@ struct LineCtx {
         if (S::BULK && old1 && !(a.skip & 2)) {
             mbar_arrive_expect_tx(bar + 1, S::TILE_BYTES);
             for (int i = 0; i < S::BULK_PARTS; i++)
-                bulk_copy_g2s(pf1 + i * PART2, a.st1 + tbase + i * PART2, PART, bar + 1);
+                bulk_copy_g2s_once<STREAM>(pf1 + i * PART2, a.st1 + tbase + i * PART2, PART, bar + 1);
         }
         if (S::BULK && old2 && !(a.skip & 4)) {
             mbar_arrive_expect_tx(bar + 2, S::TILE_BYTES);
             for (int i = 0; i < S::BULK_PARTS; i++)
-                bulk_copy_g2s(pf2 + i * PART2, a.st2 + tbase + i * PART2, PART, bar + 2);
+                bulk_copy_g2s_once<STREAM>(pf2 + i * PART2, a.st2 + tbase + i * PART2, PART, bar + 2);
         }
     }
     // without bulk copies (!S::BULK): every thread's share of one old state tile as 16-byte cp.async
@@ -456,10 +463,11 @@ struct LineCtx {
         static_assert(NCH % S::NT == 0, "tile chunks per thread");
         if (on) {
             const float2* src = st + tbase;
+            const unsigned long long pol = STREAM ? evict_first() : 0;
 #pragma unroll
             for (int q = 0; q < NCH / S::NT; q++) {
                 const int e = 2 * ((int)threadIdx.x + q * S::NT);
-                cp_async16(pf + e, src + e);
+                cp_async16_once<STREAM>(pf + e, src + e, pol);
             }
         }
         cp_async_commit();
@@ -527,12 +535,12 @@ struct LineCtx {
     }
 };
 
-template <int L, int AX>
+template <int L, int AX, bool STREAM>
 __global__ void __launch_bounds__(LS<L>::NT, LS<L>::MINB) line_pass_kernel(LineArgs a) {
     using S = LS<L>;
     constexpr int A = S::A, B = S::B;
     extern __shared__ float4 smem_raw[];
-    LineCtx<L, AX> c(a, reinterpret_cast<float2*>(smem_raw));
+    LineCtx<L, AX, STREAM> c(a, reinterpret_cast<float2*>(smem_raw));
     const bool late = (a.flags & LF_LATE_WAIT) != 0;
     if (!late) pdl_wait();
     if (!(a.flags & (LF_TRIGGER_MID | LF_TRIGGER_END))) pdl_trigger();
@@ -646,9 +654,12 @@ template <int L>
 LineKernels make_line_kernels() {
     using S = LS<L>;
     LineKernels k;
-    k.pass[0] = line_pass_kernel<L, 0>;
-    k.pass[1] = line_pass_kernel<L, 1>;
-    k.pass[2] = line_pass_kernel<L, 2>;
+    k.pass[0][0] = line_pass_kernel<L, 0, false>;
+    k.pass[0][1] = line_pass_kernel<L, 1, false>;
+    k.pass[0][2] = line_pass_kernel<L, 2, false>;
+    k.pass[1][0] = line_pass_kernel<L, 0, true>;
+    k.pass[1][1] = line_pass_kernel<L, 1, true>;
+    k.pass[1][2] = line_pass_kernel<L, 2, true>;
     k.smem = S::smem;
     k.tc = S::TC;
     k.nt = S::NT;

@@ -78,12 +78,14 @@ cudaError_t configure_kernels(const Geom& g, int kind) {
     PAT_CFG(cudaFuncSetAttribute(zk.inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zk.smem), "zfft_inv smem");
     for (int ax = 0; ax < 3; ax++) {
         LineKernels lk = line_kernels_for(g.len[ax]);
-        if (!lk.pass[ax]) {
-            g_config_what = "no line kernel for this axis length";
-            return cudaErrorInvalidValue;
+        for (int stream = 0; stream < 2; stream++) {
+            if (!lk.pass[stream][ax]) {
+                g_config_what = "no line kernel for this axis length";
+                return cudaErrorInvalidValue;
+            }
+            PAT_CFG(cudaFuncSetAttribute(lk.pass[stream][ax], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lk.smem),
+                    "line pass smem");
         }
-        PAT_CFG(cudaFuncSetAttribute(lk.pass[ax], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lk.smem),
-                "line pass smem");
     }
     PAT_CFG(configure_sampling(g, kind), "sampling smem");
 #undef PAT_CFG
@@ -147,9 +149,21 @@ static cudaError_t launch_z(ZKernel k, const ZKernels& zk, const ZArgs& a, cudaS
     return cudaLaunchKernelEx(&cfg, k, a);
 }
 
+// Whether a step's working set (states, two spectra, kappa) is beyond what stays in the 129 MB L2 from one step to
+// the next.  Measured with evict-first states against plain ones: 39 MB (64x128x128) 0.7 % slower, 71 MB (two
+// volumes) and 77 MB (128^3) 0.3 - 1 % slower, 104 MB (three volumes) 4 % faster, 137 MB (four) 7 %, 154 MB
+// (64x256x256) 8 % and 307 MB (128x256x256) 6 % faster.
+static int states_streamed(const Geom& g) {
+    size_t b = 2 * (size_t)g.B * g.nspec * sizeof(float2);
+    for (int ax = 0; ax < 3; ax++)
+        b += (size_t)g.len[ax] * g.ntile[ax] * g.tc[ax] * (2 * (size_t)g.B * sizeof(float2) + sizeof(float));
+    return b > ((size_t)90 << 20);
+}
+
 static cudaError_t launch_line(int ax, const LineArgs& a, cudaStream_t st) {
     const LineKernels lk = line_kernels_for(a.g.len[ax]);
-    if (!lk.pass[ax]) return cudaErrorInvalidValue;
+    const LineKernel kernel = lk.pass[states_streamed(a.g)][ax];
+    if (!kernel) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((a.ncols + lk.tc - 1) / lk.tc, a.g.B, 1);
     cfg.blockDim = dim3(lk.nt, 1, 1);
@@ -158,7 +172,7 @@ static cudaError_t launch_line(int ax, const LineArgs& a, cudaStream_t st) {
     cudaLaunchAttribute attr[1] = {pdl_attr()};
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, lk.pass[ax], a);
+    return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
 static const int kLineClass[3] = {KC_LINE_Z, KC_LINE_Y, KC_LINE_X};
