@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <string>
 
+#include "pat_fft.cuh"
 #include "pat_internal.h"
 
 namespace pat {
@@ -110,13 +111,18 @@ struct TvStep {
     long long n, N;   // voxels per image, B * n
 };
 
-__device__ __forceinline__ void tv_project(float& a, float& b, float& e, float alpha) {
-    const float nrm = sqrtf(a * a + b * b + e * e);
-    const float s = (nrm > alpha) ? alpha / nrm : 1.f;
-    a *= s;
-    b *= s;
-    e *= s;
+// The projection of the dual (a, b, e) onto the ball of radius alpha multiplies it by tv_scale(its squared norm).
+__device__ __forceinline__ float tv_scale(float n, float alpha) {
+    const float g = sqrtf(n);
+    return (g > alpha) ? alpha / g : 1.f;
 }
+
+// The squared norm.  Lines are cut into pieces of 32 voxels, and the dual of a piece's last voxel enters the
+// voxel after it with the first two squares added the other way round (tv_square_seam).  Both kernels do so: the
+// solver's restarts amplify a last bit of the prox to 1e-8 of its residuals, and a solve has to come out the same
+// whichever kernel a length, an alignment or an odd iteration picks.
+__device__ __forceinline__ float tv_square(float a, float b, float e) { return fmaf(e, e, fmaf(a, a, b * b)); }
+__device__ __forceinline__ float tv_square_seam(float a, float b, float e) { return fmaf(e, e, fmaf(b, b, a * a)); }
 
 // what a thread reads for plane z (its qbar at z itself is carried from the plane before)
 struct TvIn {
@@ -184,15 +190,17 @@ __global__ void __launch_bounds__(32 * kTvWarps) tv_step_kernel(TvStep a) {
         const float gy = yn ? qyn - qc : 0.f;
         const float gx = xn ? (lane < 31 ? qxn : cur.qr) - qc : 0.f;
         float dz = fmaf(a.sigma, gz, cur.xz), dy = fmaf(a.sigma, gy, cur.xy), dx = fmaf(a.sigma, gx, cur.xx);
-        tv_project(dz, dy, dx, a.alpha);
+        const float s = tv_scale(tv_square(dz, dy, dx), a.alpha);
+        dz *= s;
+        dy *= s;
+        dx *= s;
         // new dual at x0 - 1 (lane 0 of the output rows): only its x component is used
         float dlx = 0.f;
         if (halo) {
             float ez = fmaf(a.sigma, zn ? cur.qln - qlc : 0.f, cur.lz);
             float ey = fmaf(a.sigma, yn ? cur.qld - qlc : 0.f, cur.ly);
             float ex = fmaf(a.sigma, qc - qlc, cur.lx);
-            tv_project(ez, ey, ex, a.alpha);
-            dlx = ex;
+            dlx = ex * tv_scale(tv_square_seam(ez, ey, ex), a.alpha);
         }
         sy[w][lane] = dy;
         __syncthreads();
@@ -218,6 +226,220 @@ __global__ void __launch_bounds__(32 * kTvWarps) tv_step_kernel(TvStep a) {
         qlc = cur.qln;
     };
     for (int z = zs; z < z1; z++) step(z, load(z));
+}
+
+// Two primal-dual iterations per launch.  One iteration moves 44 bytes per voxel for about 90 instructions; at
+// 128x256x256, where the fields do not fit the L2, that was 105 us against 55 us of memory time, and at
+// 64x128x128, where they do, 15.7 us of latency between barriers.  Fused, the fields are read and written once
+// per two iterations.  A CTA owns rows y0 .. y0 + H - 1 (and 128 columns x of lines longer than that) over a run
+// of z planes and marches along z; a thread holds four consecutive x of one row.  At plane z it evaluates
+// the first iteration's dual and primal there and the second iteration's for plane z - 1, which needs the first
+// one's over-relaxed iterate at z.  What the second iteration reads of neighbouring tiles is evaluated
+// redundantly: duals of rows y0 - 2 .. y0 + H and y0 - 1 .. y0 + H - 1, primals one row less (at H = 8: 20
+// and 18 rows for 16), and three planes more than a run stores.  Neighbours along x and y come through
+// shared memory (two barriers per plane for both iterations), along z through registers; a plane's inputs
+// are fetched while the one before is computed.  Per voxel the operations are tv_step_kernel's, in the same
+// order, so the results are the same bit for bit.  20 iterations of 128x256x256 2193 -> 1113 us,
+// 50 of 64x128x128 829 -> 425 us.
+struct TvStep2 {
+    const float* qb_in;
+    float* qb_out;
+    const float* xi_in;  // components z, y, x at offsets 0, N, 2N
+    float* xi_out;
+    const float* q_in;
+    float* q_out;
+    const float* p;
+    float alpha;
+    float sigma[2], tau[2], theta[2], inv[2];  // inv = 1 / (1 + tau)
+    int nonneg;
+    int nz, ny, nx;
+    int ntx, H, split;   // threads per row, rows stored per tile; split: lines longer than a tile
+    int zrun, nruns;     // planes per run, runs per image
+    long long n, N;      // voxels per image, B * n
+};
+constexpr int kTv2Cols = 128;     // columns a tile stores when lines are split (one more thread on each side)
+constexpr int kTv2Threads = 384;  // most threads of a CTA
+
+struct TvIn4 {
+    float4 qn, qy;      // qbar at z + 1, at y + 1
+    float qx;           // qbar at the x after the last of this thread's
+    float4 xz, xy, xx;  // dual
+    float4 q, p;
+};
+
+// tv_scale and v / d of the two-iteration kernel, which is bound by its instructions: the IEEE square root and
+// divisions were half of an iteration's 253 per voxel.  Here the root and both quotients come from one
+// reciprocal square root (and inv = 1 / d from the host) and are rounded through fma corrections: the residual of
+// a root or quotient is exact in fma, and one correction by it gives the rounded value (P. Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000", 1990).  Compared with sqrtf and the division
+// on the device: equal for all 2^24 mantissas and for 2^32 random quotients (12 differ without the step on
+// 1 / g, for 2 % of the time).  The bounds on the radius keep the residuals' exponents in range for every norm
+// that is scaled.  The norm comes out as NaN where its square is 0, infinite or NaN, of which the infinite one
+// scales by 0 and the others by 1, as in tv_scale.
+constexpr float kTvRadiusMin = 1e-15f, kTvRadiusMax = 1e15f;  // outside, or NaN: one iteration at a time
+__device__ __forceinline__ float tv_scale_fast(float n, float alpha) {
+    float r = rsqrtf(n), h = 0.5f * r, g = n * r;
+    const float t = fmaf(-g, h, 0.5f);
+    g = fmaf(g, t, g);
+    h = fmaf(h, t, h);
+    g = fmaf(fmaf(-g, g, n), h, g);      // sqrt(n)
+    r = h + h;
+    r = fmaf(r, fmaf(-g, r, 1.f), r);    // 1 / g
+    float s = alpha * r;
+    s = fmaf(fmaf(-s, g, alpha), r, s);  // alpha / g
+    s = (g > alpha) ? s : 1.f;
+    return (n > 3.402823466e38f) ? 0.f : s;
+}
+__device__ __forceinline__ float tv_divide(float v, float d, float inv) {
+    const float q = v * inv, rem = fmaf(-q, d, v);
+    return rem == rem ? fmaf(rem, inv, q) : q;  // infinite v
+}
+
+__device__ __forceinline__ float& at4(float4& v, int i) { return reinterpret_cast<float*>(&v)[i]; }
+__device__ __forceinline__ float at4(const float4& v, int i) { return reinterpret_cast<const float*>(&v)[i]; }
+
+__global__ void __launch_bounds__(kTv2Threads, 1) tv_step2_kernel(TvStep2 a) {
+    extern __shared__ float4 tv_smem[];
+    const int rows = a.H + 3, ntx = a.ntx;
+    // [row][thread]: y components of both duals, the over-relaxed iterate of two planes, and the x component of
+    // each thread's last voxel
+    float4* sdy1 = tv_smem;
+    float4* sdy2 = sdy1 + rows * ntx;
+    float4* sqb = sdy2 + rows * ntx;  // two planes
+    float* sdx1 = reinterpret_cast<float*>(sqb + 2 * rows * ntx);
+    float* sdx2 = sdx1 + rows * ntx;
+    const int rr = threadIdx.x / ntx, tx = threadIdx.x - rr * ntx;
+    const int me = threadIdx.x;  // rr * ntx + tx
+    const int x = (a.split ? (int)blockIdx.x * kTv2Cols - 4 : 0) + 4 * tx;
+    const int y = (int)blockIdx.y * a.H - 2 + rr;
+    const int b = blockIdx.z / a.nruns, run = blockIdx.z - b * a.nruns;
+    const int z0 = run * a.zrun, z1 = min(z0 + a.zrun, a.nz);
+    const bool in = x >= 0 && x < a.nx && y >= 0 && y < a.ny;
+    const bool own = in && rr >= 2 && rr < a.H + 2 && (!a.split || (tx > 0 && tx < ntx - 1));
+    const bool yn = y + 1 < a.ny, xlast = x + 4 >= a.nx;  // the last of the four has no successor
+    const bool seam = (x & 31) == 28;                     // the last of the four ends a piece of the line
+    const float inside = a.alpha * a.alpha * 0.99999f;    // squared norms up to here are not scaled
+    const bool upy = rr + 1 < rows;                       // row y + 1 is in the tile
+    const long long plane = (long long)a.ny * a.nx;
+    const long long base = b * a.n + (long long)y * a.nx + x;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    // through L2: written by the launch before, which may still run when this one starts
+    auto ld = [](const float* p) { return __ldcg(reinterpret_cast<const float4*>(p)); };
+    auto load = [&](int z) {
+        TvIn4 v;
+        const long long o = base + z * plane;
+        const bool on = in && z < a.nz;
+        v.qn = (on && z + 1 < a.nz) ? ld(a.qb_in + o + plane) : zero;
+        v.qy = (on && yn) ? ld(a.qb_in + o + a.nx) : zero;
+        v.qx = (on && !xlast) ? __ldcg(a.qb_in + o + 4) : 0.f;
+        v.xz = on ? ld(a.xi_in + o) : zero;
+        v.xy = on ? ld(a.xi_in + a.N + o) : zero;
+        v.xx = on ? ld(a.xi_in + 2 * a.N + o) : zero;
+        v.q = on ? ld(a.q_in + o) : zero;
+        v.p = on ? ld(a.p + o) : zero;
+        return v;
+    };
+    // new dual of four voxels from (dz, dy, dx) and qbar at them, at z + 1, y + 1 and the x after the last; dxr is
+    // the last one's x component as it enters the voxel after it
+    auto dual = [&](float sigma, bool zn, const float4& qc, const float4& qn, const float4& qy, float qx, float4& dz,
+                    float4& dy, float4& dx, float& dxr) {
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const float c = at4(qc, i), r = i < 3 ? at4(qc, i + 1) : qx;
+            const float gz = zn ? at4(qn, i) - c : 0.f;
+            const float gy = yn ? at4(qy, i) - c : 0.f;
+            const float gx = (i < 3 || !xlast) ? r - c : 0.f;
+            float ez = fmaf(sigma, gz, at4(dz, i)), ey = fmaf(sigma, gy, at4(dy, i)), ex = fmaf(sigma, gx, at4(dx, i));
+            const float n = tv_square(ez, ey, ex), s = tv_scale_fast(n, a.alpha);
+            at4(dz, i) = ez * s;
+            at4(dy, i) = ey * s;
+            at4(dx, i) = ex * s;
+            if (i == 3) {
+                const float ns = tv_square_seam(ez, ey, ex);
+                float ss = s;
+                if (seam && ns != n && ns > inside) ss = tv_scale_fast(ns, a.alpha);  // else the same
+                dxr = ex * ss;
+            }
+        }
+    };
+    // new primal and over-relaxed iterate from the new dual, its z component at z - 1, y component at y - 1 and x
+    // component at the x before the first
+    auto primal = [&](int k, int z, const float4& q, const float4& p, const float4& dz, const float4& pz, const float4& dy,
+                      const float4& dyl, const float4& dx, float dxl, float4& qn, float4& qb) {
+        const float tau = a.tau[k], theta = a.theta[k];
+        const bool zn = z + 1 < a.nz;
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            float gt = 0.f;
+            if (zn) gt -= at4(dz, i);
+            if (z > 0) gt += at4(pz, i);
+            if (yn) gt -= at4(dy, i);
+            if (y > 0) gt += at4(dyl, i);
+            if (i < 3 || !xlast) gt -= at4(dx, i);
+            if (i > 0 || x > 0) gt += i > 0 ? at4(dx, i - 1) : dxl;
+            float v = tv_divide(fmaf(-tau, gt, fmaf(tau, at4(p, i), at4(q, i))), 1.f + tau, a.inv[k]);
+            if (a.nonneg) v = fmaxf(0.f, v);
+            at4(qn, i) = v;
+            at4(qb, i) = fmaf(theta, v - at4(q, i), v);
+        }
+    };
+    const int up = me + ntx, down = me - ntx;  // rows y + 1, y - 1
+    pdl_wait();     // the launch before, whose results these are, is complete
+    pdl_trigger();  // the next one may be set up while this one runs
+    const int zs = z0 > 1 ? z0 - 2 : 0;
+    float4 qc = in ? ld(a.qb_in + base + zs * plane) : zero;  // qbar at z
+    float4 pz1 = zero, pz2 = zero;                            // z component of the duals a plane before
+    float4 d1z = zero, d1y = zero, d1x = zero;                // first dual, iterate and input at z - 1
+    float4 q1 = zero, qb1 = zero, p1 = zero;
+    TvIn4 cur = load(zs);
+    for (int z = zs; z <= z1; z++) {
+        const TvIn4 nxt = load(z + 1 <= z1 ? z + 1 : a.nz);
+        float4 dz = cur.xz, dy = cur.xy, dx = cur.xx;
+        dual(a.sigma[0], z + 1 < a.nz, qc, cur.qn, cur.qy, cur.qx, dz, dy, dx, sdx1[me]);
+        sdy1[me] = dy;
+        __syncthreads();
+        // first primal at z
+        float4 qn, qb;
+        {
+            const float4 dyl = rr > 0 ? sdy1[down] : zero;
+            const float dxl = tx > 0 ? sdx1[me - 1] : 0.f;
+            primal(0, z, cur.q, cur.p, dz, pz1, dy, dyl, dx, dxl, qn, qb);
+        }
+        float4* sq = sqb + (z & 1) * rows * ntx;
+        sq[me] = qb;
+        // second dual at z - 1 (from the second plane on; its neighbours were stored a plane ago)
+        float4 ez = d1z, ey = d1y, ex = d1x;
+        if (z > zs) {
+            const float4* so = sqb + ((z - 1) & 1) * rows * ntx;
+            const float4 qy = upy ? so[up] : zero;
+            const float qx = tx + 1 < ntx ? so[me + 1].x : 0.f;
+            dual(a.sigma[1], z < a.nz, qb1, qb, qy, qx, ez, ey, ex, sdx2[me]);
+        }
+        sdy2[me] = ey;
+        __syncthreads();
+        // second primal at z - 1
+        if (own && z - 1 >= z0) {
+            float4 q2, qb2;
+            primal(1, z - 1, q1, p1, ez, pz2, ey, sdy2[down], ex, tx > 0 ? sdx2[me - 1] : 0.f, q2, qb2);
+            const long long o = base + (z - 1) * plane;
+            auto st = [](float* p, const float4& v) { *reinterpret_cast<float4*>(p) = v; };
+            st(a.q_out + o, q2);
+            st(a.qb_out + o, qb2);
+            st(a.xi_out + o, ez);
+            st(a.xi_out + a.N + o, ey);
+            st(a.xi_out + 2 * a.N + o, ex);
+        }
+        pz1 = dz;
+        pz2 = ez;
+        d1z = dz;
+        d1y = dy;
+        d1x = dx;
+        q1 = qn;
+        qb1 = qb;
+        p1 = cur.p;
+        qc = cur.qn;
+        cur = nxt;
+    }
 }
 
 // ------------------------------------------------------------------------------ FP64 reductions
@@ -324,6 +546,7 @@ static pat_status ensure_ws(pat_grid* G, bool solver) {
         if (st == PAT_OK) st = grid_alloc(G, (void**)&w.xi, 3 * N * sizeof(float), "prox dual");
         if (st == PAT_OK) st = grid_alloc(G, (void**)&w.xi2, 3 * N * sizeof(float), "prox dual");
         if (st == PAT_OK) st = grid_alloc(G, (void**)&w.z, N * sizeof(float), "prox input copy");
+        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.q2, N * sizeof(float), "prox iterate");
         if (st == PAT_OK) st = grid_alloc(G, (void**)&w.partial, kRedBlocks * sizeof(double), "reduction");
         if (st == PAT_OK) st = grid_alloc(G, (void**)&w.result, sizeof(double), "reduction");
         if (st == PAT_OK) {
@@ -350,12 +573,45 @@ static pat_status ensure_ws(pat_grid* G, bool solver) {
     return PAT_OK;
 }
 
+// Tiling of tv_step2_kernel: rows per tile so that a CTA has up to kTv2Threads threads, and the z run that
+// minimises rounds of CTAs times planes marched (a run evaluates three planes more than it stores).
+static void tv2_plan(const TvDims& d, int B, TvStep2* a, dim3* grid, int* threads, size_t* smem) {
+    a->split = d.nx > kTv2Cols;
+    a->ntx = a->split ? kTv2Cols / 4 + 2 : d.nx / 4;
+    int H = 16;
+    while (H > 8 && (H + 3) * a->ntx > kTv2Threads) H /= 2;
+    if (H > d.ny) H = d.ny;
+    a->H = H;
+    const int gx = a->split ? (d.nx + kTv2Cols - 1) / kTv2Cols : 1, gy = (d.ny + H - 1) / H;
+    const long long tiles = (long long)gx * gy * B;
+    *threads = (H + 3) * a->ntx;
+    const int resident = 152 * std::max(1, kTv2Threads / *threads);
+    long long best = 0;
+    for (int run = 1; run <= d.nz; run++) {
+        const int n = (d.nz + run - 1) / run;
+        if ((long long)B * n > 65535) continue;  // grid's z extent
+        const long long cost = ((tiles * n + resident - 1) / resident) * (run + 3);
+        if (best == 0 || cost < best) {
+            best = cost;
+            a->zrun = run;
+            a->nruns = n;
+        }
+    }
+    *grid = dim3(gx, gy, B * a->nruns);
+    *smem = (size_t)*threads * (4 * sizeof(float4) + 2 * sizeof(float));
+}
+
 // PDHG for the positivity-constrained TV denoising problem; q (output) must not alias p.
 static pat_status tv_prox_run(Ctx& c, const float* p, float* q, double alpha, int iters, int nonneg) {
     SolverWs& w = c.G->sw;
     const int nb = ew_blocks(c.N);
-    clamp_copy_kernel<<<nb, 256, 0, c.st>>>(q, w.qbar, p, c.N);
-    if (!nonneg) PAT_CUDA(cudaMemcpyAsync(q, p, c.N * sizeof(float), cudaMemcpyDeviceToDevice, c.st), "prox init");
+    // iterations two at a time (16-byte accesses; a caller's image may be aligned to less)
+    const bool vec = (((uintptr_t)p | (uintptr_t)q) & 15) == 0;
+    const int pairs = vec && alpha >= kTvRadiusMin && alpha <= kTvRadiusMax ? iters / 2 : 0;
+    // pairs of iterations read one iterate buffer and write the other, the last one q
+    float* qbuf[2] = {(pairs & 1) ? w.q2 : q, (pairs & 1) ? q : w.q2};
+    clamp_copy_kernel<<<nb, 256, 0, c.st>>>(qbuf[0], w.qbar, p, c.N);
+    if (!nonneg) PAT_CUDA(cudaMemcpyAsync(qbuf[0], p, c.N * sizeof(float), cudaMemcpyDeviceToDevice, c.st), "prox init");
     if (!nonneg) PAT_CUDA(cudaMemcpyAsync(w.qbar, p, c.N * sizeof(float), cudaMemcpyDeviceToDevice, c.st), "prox init");
     if (alpha <= 0.0 || iters == 0) {
         PAT_CUDA(cudaGetLastError(), "prox launch");
@@ -364,41 +620,86 @@ static pat_status tv_prox_run(Ctx& c, const float* p, float* q, double alpha, in
     PAT_CUDA(cudaMemsetAsync(w.xi, 0, 3 * c.N * sizeof(float), c.st), "prox init");
     const TvDims& d = c.td;
     const int B = (int)(d.total / d.n);
-    const int gx = (d.nx + 31) / 32, gy = (d.ny + kTvRows - 1) / kTvRows;
-    // runs of z planes: about 512 CTAs in all, at least 4 planes per run (each run evaluates one
-    // plane more than it stores)
-    const long long cols = (long long)gx * gy * B;
-    int nruns = (int)std::max<long long>(1, std::min<long long>((512 + cols - 1) / cols, (d.nz + 3) / 4));
-    const int zrun = (d.nz + nruns - 1) / nruns;
-    nruns = (d.nz + zrun - 1) / zrun;
-    TvStep a;
-    a.q = q;
-    a.p = p;
-    a.alpha = (float)alpha;
-    a.nonneg = nonneg;
-    a.nz = d.nz;
-    a.ny = d.ny;
-    a.nx = d.nx;
-    a.zrun = zrun;
-    a.nruns = nruns;
-    a.n = (long long)d.n;
-    a.N = (long long)d.total;
-    const dim3 grid(gx, gy, B * nruns);
     float* qb[2] = {w.qbar, w.qbar2};
     float* xi[2] = {w.xi, w.xi2};
     double tau = 1.0 / sqrt(12.0), sigma = 1.0 / (tau * 12.0);
-    for (int it = 0; it < iters; it++) {
+    auto next = [&](float* sg, float* ta, float* th) {
         const double theta = 1.0 / sqrt(1.0 + 2.0 * tau);
-        a.qb_in = qb[it & 1];
-        a.qb_out = qb[(it + 1) & 1];
-        a.xi_in = xi[it & 1];
-        a.xi_out = xi[(it + 1) & 1];
-        a.sigma = (float)sigma;
-        a.tau = (float)tau;
-        a.theta = (float)theta;
-        tv_step_kernel<<<grid, 32 * kTvWarps, 0, c.st>>>(a);
+        *sg = (float)sigma;
+        *ta = (float)tau;
+        *th = (float)theta;
         tau *= theta;
         sigma /= theta;
+    };
+    if (pairs > 0) {
+        TvStep2 a = {};
+        dim3 grid;
+        int threads;
+        size_t smem;
+        tv2_plan(d, B, &a, &grid, &threads, &smem);
+        a.p = p;
+        a.alpha = (float)alpha;
+        a.nonneg = nonneg;
+        a.nz = d.nz;
+        a.ny = d.ny;
+        a.nx = d.nx;
+        a.n = (long long)d.n;
+        a.N = (long long)d.total;
+        for (int it = 0; it < pairs; it++) {
+            const int in = it & 1, out = in ^ 1;
+            a.qb_in = qb[in];
+            a.qb_out = qb[out];
+            a.xi_in = xi[in];
+            a.xi_out = xi[out];
+            a.q_in = qbuf[in];
+            a.q_out = qbuf[out];
+            for (int k = 0; k < 2; k++) {
+                next(&a.sigma[k], &a.tau[k], &a.theta[k]);
+                a.inv[k] = 1.f / (1.f + a.tau[k]);
+            }
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = grid;
+            cfg.blockDim = dim3(threads);
+            cfg.dynamicSmemBytes = smem;
+            cfg.stream = c.st;
+            cudaLaunchAttribute at;
+            at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at.val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            PAT_CUDA(cudaLaunchKernelEx(&cfg, tv_step2_kernel, a), "prox launch");
+        }
+    }
+    // what is left (an odd iteration; all of them for unaligned images) one at a time, in place on q
+    if (2 * pairs < iters) {
+        const int gx = (d.nx + 31) / 32, gy = (d.ny + kTvRows - 1) / kTvRows;
+        // runs of z planes: about 512 CTAs in all, at least 4 planes per run (each run evaluates one
+        // plane more than it stores)
+        const long long cols = (long long)gx * gy * B;
+        int nruns = (int)std::max<long long>(1, std::min<long long>((512 + cols - 1) / cols, (d.nz + 3) / 4));
+        const int zrun = (d.nz + nruns - 1) / nruns;
+        nruns = (d.nz + zrun - 1) / zrun;
+        TvStep a;
+        a.q = q;
+        a.p = p;
+        a.alpha = (float)alpha;
+        a.nonneg = nonneg;
+        a.nz = d.nz;
+        a.ny = d.ny;
+        a.nx = d.nx;
+        a.zrun = zrun;
+        a.nruns = nruns;
+        a.n = (long long)d.n;
+        a.N = (long long)d.total;
+        for (int it = 2 * pairs; it < iters; it++) {
+            const int in = (it - pairs) & 1;  // buffers alternate per launch
+            a.qb_in = qb[in];
+            a.qb_out = qb[in ^ 1];
+            a.xi_in = xi[in];
+            a.xi_out = xi[in ^ 1];
+            next(&a.sigma, &a.tau, &a.theta);
+            tv_step_kernel<<<dim3(gx, gy, B * nruns), 32 * kTvWarps, 0, c.st>>>(a);
+        }
     }
     PAT_CUDA(cudaGetLastError(), "prox launch");
     return PAT_OK;
