@@ -10,6 +10,7 @@
 #include <string>
 
 #include "../../include/pat_unet.h"
+#include "pat_fft.cuh"
 #include "pat_internal.h"
 
 namespace pat {
@@ -25,6 +26,9 @@ cudaError_t wgrad_tc(const void* x, int ldx, int cin, const void* dy, int ldy, i
 namespace {
 
 typedef __nv_bfloat16 bf16;
+using pat::launch_pdl;
+using pat::pdl_trigger;
+using pat::pdl_wait;
 
 
 __global__ void cast_weights_kernel(const float* __restrict__ w32, int cin, int cout, bf16* __restrict__ wb,
@@ -43,12 +47,14 @@ __global__ void cast_weights_kernel(const float* __restrict__ w32, int cin, int 
 // the network), and a scalar form for anything else.  One thread per channel with a 64-bit division and 2-byte
 // accesses, they ran at a tenth of the memory bandwidth (up 132 us, ReLU backward 43, pool backward 79 at
 // 64x128x128 voxels); the vector forms are bound by memory.  MASK: the gradient is also taken through the
-// ReLU whose output is y (zero where y is not positive), which saves a pass of its own.
+// ReLU whose output is y (zero where y is not positive), which saves a pass of its own.  The vector forms are
+// launched with programmatic stream serialisation, as the convolutions are (pat_unet_tc.cu).
 
 struct V8 {
     uint4 u;
 };
-__device__ __forceinline__ V8 ld8(const bf16* p) { return V8{*reinterpret_cast<const uint4*>(p)}; }
+// (through L2: written by the kernel before, which may still run when this one starts)
+__device__ __forceinline__ V8 ld8(const bf16* p) { return V8{__ldcg(reinterpret_cast<const uint4*>(p))}; }
 __device__ __forceinline__ void st8(bf16* p, V8 v) { *reinterpret_cast<uint4*>(p) = v.u; }
 __device__ __forceinline__ void unpack8(V8 v, float* f) {
     const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&v.u);
@@ -113,6 +119,8 @@ __global__ void relu_bwd_kernel(bf16* __restrict__ g, int ldg, const bf16* __res
 // D, H, W: the pooled (small) volume
 __global__ void __launch_bounds__(256) pool8_kernel(const bf16* __restrict__ x, int ldx, unsigned c8, unsigned H, unsigned W,
                                                     bf16* __restrict__ y, int ldy, unsigned n) {
+    pdl_wait();
+    pdl_trigger();
     for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
         const Vox e = vox_of(i, c8);
         const unsigned c0 = child0(e.v, H, W);
@@ -152,6 +160,8 @@ __global__ void pool_kernel(const bf16* __restrict__ x, int ldx, int C, int D, i
 __global__ void __launch_bounds__(256) pool_bwd_add8_kernel(const bf16* __restrict__ dy, int ldd, unsigned c8, unsigned H,
                                                             unsigned W, bf16* __restrict__ dx, int ldx,
                                                             const bf16* __restrict__ mask, int ldm, unsigned n) {
+    pdl_wait();
+    pdl_trigger();
     for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
         const Vox e = vox_of(i, c8);
         const unsigned c0 = child0(e.v, H, W);
@@ -193,6 +203,8 @@ __global__ void pool_bwd_add_kernel(const bf16* __restrict__ dy, int ldd, int C,
 // D, H, W: the small volume
 __global__ void __launch_bounds__(256) up8_kernel(const bf16* __restrict__ x, int ldx, unsigned c8, unsigned H, unsigned W,
                                                   bf16* __restrict__ y, int ldy, unsigned n) {
+    pdl_wait();
+    pdl_trigger();
     for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
         const Vox e = vox_of(i, c8);
         const unsigned c0 = child0(e.v, H, W);
@@ -216,6 +228,8 @@ __global__ void up_kernel(const bf16* __restrict__ x, int ldx, int C, int D, int
 __global__ void __launch_bounds__(256) up_bwd8_kernel(const bf16* __restrict__ dy, int ldd, unsigned c8, unsigned H,
                                                       unsigned W, bf16* __restrict__ dx, int ldx,
                                                       const bf16* __restrict__ mask, int ldm, unsigned n) {
+    pdl_wait();
+    pdl_trigger();
     for (unsigned i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) {
         const Vox e = vox_of(i, c8);
         const unsigned c0 = child0(e.v, H, W);
@@ -252,9 +266,11 @@ __global__ void up_bwd_kernel(const bf16* __restrict__ dy, int ldd, int C, int D
 
 // two 16-byte halves of a voxel's 16 channels per thread pair: consecutive threads write consecutive bytes
 __global__ void __launch_bounds__(256) input8_kernel(const float* __restrict__ xin, float s, long long n, bf16* __restrict__ x16) {
+    pdl_wait();
+    pdl_trigger();
     for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += gridDim.x * 256LL) {
         float f[8] = {};
-        if (!(i & 1)) f[0] = s * xin[i >> 1];
+        if (!(i & 1)) f[0] = s * __ldcg(xin + (i >> 1));
         st8(x16 + 8 * i, pack8(f));
     }
 }
@@ -267,9 +283,11 @@ __global__ void input_kernel(const float* __restrict__ xin, float s, long long V
 
 __global__ void __launch_bounds__(256) head8_kernel(const bf16* __restrict__ h, const float* __restrict__ head, long long V,
                                                     float* __restrict__ out) {
+    pdl_wait();
+    pdl_trigger();
     float w[17];
 #pragma unroll
-    for (int c = 0; c < 17; c++) w[c] = __ldg(head + c);
+    for (int c = 0; c < 17; c++) w[c] = __ldca(head + c);
     for (long long v = blockIdx.x * 256LL + threadIdx.x; v < V; v += gridDim.x * 256LL) {
         float f[16], s = w[16];
         unpack8(ld8(h + 16 * v), f);
@@ -324,17 +342,19 @@ __global__ void __launch_bounds__(256) head_bwd8_kernel(const bf16* __restrict__
                                                         const float* __restrict__ out, const float* __restrict__ target,
                                                         long long V, bf16* __restrict__ dh, int mask,
                                                         double* __restrict__ partial) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ double red[256][18];
     FloatPair acc[18];
     float w[16];
 #pragma unroll
-    for (int c = 0; c < 16; c++) w[c] = __ldg(head + c);
+    for (int c = 0; c < 16; c++) w[c] = __ldca(head + c);
     const double gs = 2.0 / (double)V;
     for (long long v = blockIdx.x * 256LL + threadIdx.x; v < V; v += gridDim.x * 256LL) {
         float f[16];
         unpack8(ld8(h + 16 * v), f);
         unpack8(ld8(h + 16 * v + 8), f + 8);
-        const float o = out[v], t = target[v];
+        const float o = __ldcg(out + v), t = __ldcg(target + v);
         const float eh = o - t, b = eh - o, el = (o - (eh - b)) - (t + b);  // o - t = eh + el exactly
         const float g = (float)(gs * ((double)o - (double)t));
         float d[16];
@@ -380,9 +400,11 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16* __restrict__ 
 // one warp per sum: strided partial sums and a fixed-order tree
 __global__ void __launch_bounds__(576) head_bwd_final_kernel(const double* __restrict__ partial, int nb, long long V,
                                                              float* __restrict__ ghead, double* __restrict__ loss) {
+    pdl_wait();
+    pdl_trigger();
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double s = 0.0;
-    for (int b = lane; b < nb; b += 32) s += partial[(size_t)b * 18 + k];
+    for (int b = lane; b < nb; b += 32) s += __ldcg(partial + (size_t)b * 18 + k);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane) return;
     if (k < 17) ghead[k] = (float)s;
@@ -517,8 +539,8 @@ pat_status pat_unet_pool(const void* x, int32_t ldx, int32_t C, int32_t D, int32
         return bad("pat_unet_pool: bad argument (even dims >= 2)");
     const long long P = (long long)D * H * W / 8;
     if (vec8(C, ldx, ldy, 8, x, y, y, 8 * P))
-        pool8_kernel<<<grid_for(P * C / 8), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, ldx, C / 8, H / 2, W / 2,
-                                                                           (bf16*)y, ldy, (unsigned)(P * C / 8));
+        launch_pdl(pool8_kernel, grid_for(P * C / 8), 256, 0, (cudaStream_t)stream, (const bf16*)x, ldx, C / 8, H / 2, W / 2,
+                   (bf16*)y, ldy, (unsigned)(P * C / 8));
     else
         pool_kernel<<<grid_for(P * C), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, ldx, C, D, H, W, (bf16*)y, ldy);
     return launched("pat_unet_pool");
@@ -530,8 +552,8 @@ pat_status pat_unet_pool_bwd_add(const void* dy, int32_t ldd, int32_t C, int32_t
         return bad("pat_unet_pool_bwd_add: bad argument (even dims >= 2)");
     const long long P = (long long)D * H * W / 8;
     if (vec8(C, ldx, ldd, 8, dx, dy, dy, 8 * P))
-        pool_bwd_add8_kernel<<<grid_for(P * C / 8), 256, 0, (cudaStream_t)stream>>>(
-            (const bf16*)dy, ldd, C / 8, H / 2, W / 2, (bf16*)dx, ldx, nullptr, 0, (unsigned)(P * C / 8));
+        launch_pdl(pool_bwd_add8_kernel, grid_for(P * C / 8), 256, 0, (cudaStream_t)stream,
+                   (const bf16*)dy, ldd, C / 8, H / 2, W / 2, (bf16*)dx, ldx, nullptr, 0, (unsigned)(P * C / 8));
     else
         pool_bwd_add_kernel<<<grid_for(8 * P * C), 256, 0, (cudaStream_t)stream>>>((const bf16*)dy, ldd, C, D, H, W,
                                                                                   (bf16*)dx, ldx);
@@ -544,8 +566,8 @@ pat_status pat_unet_pool_bwd_add_masked(const void* dy, int32_t ldd, int32_t C, 
         return bad("pat_unet_pool_bwd_add_masked: bad argument (even dims >= 2)");
     const long long P = (long long)D * H * W / 8;
     if (vec8(C, ldx, ldd, lda, dx, dy, act, 8 * P)) {
-        pool_bwd_add8_kernel<<<grid_for(P * C / 8), 256, 0, (cudaStream_t)stream>>>(
-            (const bf16*)dy, ldd, C / 8, H / 2, W / 2, (bf16*)dx, ldx, (const bf16*)act, lda, (unsigned)(P * C / 8));
+        launch_pdl(pool_bwd_add8_kernel, grid_for(P * C / 8), 256, 0, (cudaStream_t)stream,
+                   (const bf16*)dy, ldd, C / 8, H / 2, W / 2, (bf16*)dx, ldx, (const bf16*)act, lda, (unsigned)(P * C / 8));
         return launched("pat_unet_pool_bwd_add_masked");
     }
     const pat_status s = pat_unet_pool_bwd_add(dy, ldd, C, D, H, W, dx, ldx, stream);
@@ -557,8 +579,8 @@ pat_status pat_unet_up(const void* x, int32_t ldx, int32_t C, int32_t D, int32_t
     if (!x || !y || C < 1 || ldx < C || ldy < C || D < 1 || H < 1 || W < 1) return bad("pat_unet_up: bad argument");
     const long long P = (long long)D * H * W;
     if (vec8(C, ldx, ldy, 8, x, y, y, 8 * P))
-        up8_kernel<<<grid_for(P * C / 8), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, ldx, C / 8, H, W, (bf16*)y, ldy,
-                                                                         (unsigned)(P * C / 8));
+        launch_pdl(up8_kernel, grid_for(P * C / 8), 256, 0, (cudaStream_t)stream, (const bf16*)x, ldx, C / 8, H, W, (bf16*)y,
+                   ldy, (unsigned)(P * C / 8));
     else
         up_kernel<<<grid_for(8 * P * C), 256, 0, (cudaStream_t)stream>>>((const bf16*)x, ldx, C, D, H, W, (bf16*)y, ldy);
     return launched("pat_unet_up");
@@ -569,8 +591,8 @@ pat_status pat_unet_up_bwd(const void* dy, int32_t ldd, int32_t C, int32_t D, in
     if (!dy || !dx || C < 1 || ldx < C || ldd < C || D < 1 || H < 1 || W < 1) return bad("pat_unet_up_bwd: bad argument");
     const long long P = (long long)D * H * W;
     if (vec8(C, ldx, ldd, 8, dx, dy, dy, 8 * P))
-        up_bwd8_kernel<<<grid_for(P * C / 8), 256, 0, (cudaStream_t)stream>>>(
-            (const bf16*)dy, ldd, C / 8, H, W, (bf16*)dx, ldx, nullptr, 0, (unsigned)(P * C / 8));
+        launch_pdl(up_bwd8_kernel, grid_for(P * C / 8), 256, 0, (cudaStream_t)stream,
+                   (const bf16*)dy, ldd, C / 8, H, W, (bf16*)dx, ldx, nullptr, 0, (unsigned)(P * C / 8));
     else
         up_bwd_kernel<<<grid_for(P * C), 256, 0, (cudaStream_t)stream>>>((const bf16*)dy, ldd, C, D, H, W, (bf16*)dx, ldx);
     return launched("pat_unet_up_bwd");
@@ -582,8 +604,8 @@ pat_status pat_unet_up_bwd_masked(const void* dy, int32_t ldd, int32_t C, int32_
         return bad("pat_unet_up_bwd_masked: bad argument");
     const long long P = (long long)D * H * W;
     if (vec8(C, ldx, ldd, lda, dx, dy, act, 8 * P)) {
-        up_bwd8_kernel<<<grid_for(P * C / 8), 256, 0, (cudaStream_t)stream>>>(
-            (const bf16*)dy, ldd, C / 8, H, W, (bf16*)dx, ldx, (const bf16*)act, lda, (unsigned)(P * C / 8));
+        launch_pdl(up_bwd8_kernel, grid_for(P * C / 8), 256, 0, (cudaStream_t)stream,
+                   (const bf16*)dy, ldd, C / 8, H, W, (bf16*)dx, ldx, (const bf16*)act, lda, (unsigned)(P * C / 8));
         return launched("pat_unet_up_bwd_masked");
     }
     const pat_status s = pat_unet_up_bwd(dy, ldd, C, D, H, W, dx, ldx, stream);
@@ -592,14 +614,14 @@ pat_status pat_unet_up_bwd_masked(const void* dy, int32_t ldd, int32_t C, int32_
 
 pat_status pat_unet_input(const float* xin, float s, int64_t V, void* x16, void* stream) {
     if (!xin || !x16 || V < 0) return bad("pat_unet_input: bad argument");
-    if (al16(x16)) input8_kernel<<<grid_for(V * 2), 256, 0, (cudaStream_t)stream>>>(xin, s, V * 2, (bf16*)x16);
+    if (al16(x16)) launch_pdl(input8_kernel, grid_for(V * 2), 256, 0, (cudaStream_t)stream, xin, s, V * 2, (bf16*)x16);
     else input_kernel<<<grid_for(V * 16), 256, 0, (cudaStream_t)stream>>>(xin, s, V, (bf16*)x16);
     return launched("pat_unet_input");
 }
 
 pat_status pat_unet_head(const void* h, const float* head, int64_t V, float* out, void* stream) {
     if (!h || !head || !out || V < 0) return bad("pat_unet_head: bad argument");
-    if (al16(h)) head8_kernel<<<grid_for(V), 256, 0, (cudaStream_t)stream>>>((const bf16*)h, head, V, out);
+    if (al16(h)) launch_pdl(head8_kernel, grid_for(V), 256, 0, (cudaStream_t)stream, (const bf16*)h, head, V, out);
     else head_kernel<<<grid_for(V), 256, 0, (cudaStream_t)stream>>>((const bf16*)h, head, V, out);
     return launched("pat_unet_head");
 }
@@ -614,9 +636,12 @@ static pat_status head_bwd(const char* who, const void* h, const float* head, co
     if (!h || !head || !out || !target || !dh || !ghead || !loss || !partial || V < 1)
         return bad((std::string(who) + ": bad argument").c_str());
     const cudaStream_t st = (cudaStream_t)stream;
-    const auto kernel = al16(h) && al16(dh) ? head_bwd8_kernel : head_bwd_kernel;
-    kernel<<<kHeadBlocks, 256, 0, st>>>((const bf16*)h, head, out, target, V, (bf16*)dh, mask, partial);
-    head_bwd_final_kernel<<<1, 18 * 32, 0, st>>>(partial, kHeadBlocks, V, ghead, loss);
+    if (al16(h) && al16(dh))
+        launch_pdl(head_bwd8_kernel, kHeadBlocks, 256, 0, st, (const bf16*)h, head, out, target, V, (bf16*)dh, mask,
+                   partial);
+    else
+        head_bwd_kernel<<<kHeadBlocks, 256, 0, st>>>((const bf16*)h, head, out, target, V, (bf16*)dh, mask, partial);
+    launch_pdl(head_bwd_final_kernel, 1, 18 * 32, 0, st, partial, kHeadBlocks, V, ghead, loss);
     return launched(who);
 }
 
