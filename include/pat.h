@@ -210,9 +210,9 @@ pat_status pat_bregman_solve(pat_grid* grid, const float* f_dev, const float* wa
  * bracketed by CUDA events recorded on the call's stream.  pat_profile_enable(grid, 1) starts (and
  * clears) the record; pat_profile_read waits for the recorded events, then reports per kernel class
  * its name (NUL-terminated, at most 47 characters, in names[48*i]), total device milliseconds and
- * launch count.  Classes: line_x, line_y, line_z (the time step's line passes), plane_fft, z_fft
- * (transforms outside the time loop), sample.  n_classes receives the number written
- * (<= max_classes). */
+ * launch count.  Classes: line_x, line_y, line_z (the time step's line passes), step (the three in
+ * one launch, on small grids), plane_fft, z_fft (transforms outside the time loop), sample.
+ * n_classes receives the number written (<= max_classes). */
 pat_status pat_profile_enable(pat_grid* grid, int32_t enable);
 pat_status pat_profile_read(pat_grid* grid, int32_t max_classes, char* names, double* total_ms,
                             int64_t* launches, int32_t* n_classes);

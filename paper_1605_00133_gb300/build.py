@@ -9,11 +9,11 @@ from concurrent.futures import ThreadPoolExecutor
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpat.so")
-SOURCES = ["pat_api.cu", "pat_run.cu", "pat_zpass.cu", "pat_sample.cu", "pat_solver.cu", "pat_unet.cu",
-           "pat_unet_tc.cu"] + [
+SOURCES = ["pat_step_r3.cu", "pat_step_r4.cu", "pat_api.cu", "pat_run.cu", "pat_zpass.cu", "pat_sample.cu",
+           "pat_solver.cu", "pat_unet.cu", "pat_unet_tc.cu"] + [
     f"pat_plane_nx{n}.cu" for n in (8, 16, 32, 64, 128, 256)] + [
     f"pat_line_l{n}.cu" for n in (8, 16, 32, 64, 128, 256)]
-HEADERS = ["pat_fft.cuh", "pat_internal.h", "pat_kargs.h", "pat_plane.cuh", "pat_line.cuh",
+HEADERS = ["pat_fft.cuh", "pat_internal.h", "pat_kargs.h", "pat_plane.cuh", "pat_line.cuh", "pat_step.cuh",
            os.path.join("..", "..", "include", "pat.h"), os.path.join("..", "..", "include", "pat_unet.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC"]

@@ -298,7 +298,7 @@ static size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
 // The real plane series (sampled kinds) is live only outside the time loop: the forward writes it
 // after the last step, the adjoint has consumed it (its plane spectra) before the first.  So it
 // shares its memory with the states and 3D spectra, which are live only inside the loop.
-WsLayout workspace_layout(const Geom& g, int kind) {
+WsLayout workspace_layout(const Geom& g, int kind, size_t limit) {
     const size_t B = (size_t)g.B;
     WsLayout L;
     size_t loop = 0;
@@ -311,6 +311,10 @@ WsLayout workspace_layout(const Geom& g, int kind) {
     L.rk = round256(B * (size_t)g.T * g.nplane * sizeof(float2));
     L.rec = (kind == PAT_SAMPLE_FULL) ? 0 : round256(B * (size_t)g.T * g.m_plane * sizeof(float));
     L.total = std::max(loop, L.rec) + L.rk;
+    // the parts of small grids' spectra, unless they would break the limit (the passes do without them)
+    const size_t with = std::max(loop + 4 * L.ph, L.rec) + L.rk;
+    L.parts = step_residency(g) != 0 && (limit == 0 || with <= limit);
+    if (L.parts) L.total = with;
     return L;
 }
 
@@ -320,6 +324,8 @@ void workspace_carve(const Geom& g, const WsLayout& L, unsigned char* base, Work
     for (int a = 0; a < 3; a++)
         for (int s = 0; s < 2; s++, off += L.ms[a]) w->ms[a][s] = (float2*)(base + off);
     for (int s = 0; s < 2; s++, off += L.ph) w->ph[s] = (float2*)(base + off);
+    for (int s = 0; s < 4; s++) w->part[s / 2][s % 2] = L.parts ? (float2*)(base + off + s * L.ph) : nullptr;
+    if (L.parts) off += 4 * L.ph;
     w->rec = L.rec ? (float*)base : nullptr;  // aliases the loop state, see workspace_layout
     w->rk = (float2*)(base + std::max(off, L.rec));
 }
@@ -385,8 +391,8 @@ pat_status pat_create_grid(const pat_grid_desc* desc, const pat_sampling_desc* s
     g.m_plane = M;
 
     // the workspace cap is checked on the host, before the device is touched
-    const WsLayout layout = workspace_layout(g, G->kind);
     const int64_t limit = g_ws_limit.load();
+    const WsLayout layout = workspace_layout(g, G->kind, (size_t)limit);
     if (limit > 0 && (int64_t)layout.total > limit) {
         delete G;
         return fail(PAT_ERR_OOM, "pat_create_grid: the workspace needs " + std::to_string(layout.total) +
@@ -516,7 +522,7 @@ pat_status pat_sample_adjoint(pat_grid* G, const float* f, float* pbar, int32_t 
     return PAT_OK;
 }
 
-static const char* kClassNames[KC_COUNT] = {"line_x", "line_y", "line_z", "plane_fft", "z_fft", "sample"};
+static const char* kClassNames[KC_COUNT] = {"line_x", "line_y", "line_z", "plane_fft", "z_fft", "sample", "step"};
 
 pat_status pat_get_indices(const pat_grid* G, int32_t* host_idx_or_perm, int32_t* host_rows) {
     g_err.clear();
@@ -646,7 +652,7 @@ extern "C" pat_status pat_forward_noalloc(pat_grid* G, const float* p0, float* f
     pat_status st = check_device(G);
     if (st != PAT_OK) return st;
     const Geom& g = G->g;
-    const WsLayout L = workspace_layout(g, G->kind);
+    const WsLayout L = workspace_layout(g, G->kind, PAT_NOALLOC_SCRATCH_BYTES);
     const size_t need = L.total;
     if (need > PAT_NOALLOC_SCRATCH_BYTES)
         return fail(PAT_ERR_INVALID_ARG, "pat_forward_noalloc: this grid needs " + std::to_string(need) +

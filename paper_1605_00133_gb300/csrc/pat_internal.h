@@ -95,6 +95,7 @@ struct DeviceTables {
 struct Workspace {
     float2* ms[3][2];           // per axis: state 1 (u_i | adjoint of rho_i), state 2 (rho_i | adjoint of u_i)
     float2* ph[2];              // 3D half spectra [B][nz][nxh][ny], double-buffered across passes
+    float2* part[2][2];         // small grids: the y and z parts of both (ph holds the x part); else NULL
     float2* rk;                 // plane spectra [B][T][nxh][ny]: recorded (A) or injected (A^T)
     float* rec;                 // real plane series [B][T][M] (sampled kinds); shares memory with
                                 // ms and ph, which are dead whenever it is live
@@ -111,7 +112,7 @@ struct Scalars {
 
 // Kernel classes timed by the optional profiler (CUDA events on the launching stream).
 enum KernelClass {
-    KC_LINE_X = 0, KC_LINE_Y, KC_LINE_Z, KC_PLANE_FFT, KC_Z_FFT, KC_SAMPLE, KC_COUNT
+    KC_LINE_X = 0, KC_LINE_Y, KC_LINE_Z, KC_PLANE_FFT, KC_Z_FFT, KC_SAMPLE, KC_STEP, KC_COUNT
 };
 
 // NVTX range over a scope (for tracing tools such as Nsight Systems; a no-op when none is attached):
@@ -146,11 +147,13 @@ int plane_cluster_size(int nx, int ny);
 const char* configure_failure();  // which attribute the last failed configure_kernels call set
 cudaError_t configure_kernels(const Geom& g, int kind);
 int shd_threads(int M);  // threads per plane of the Hadamard kernels (0: no kernel for this plane size)
+int step_residency(const Geom& g);  // small grids: CTAs an SM of the kernel that does a whole step (pat_step.cuh); else 0
 // workspace layout: bytes of each part (256-byte aligned) for a grid and sampling kind
 struct WsLayout {
     size_t ms[3], ph, rk, rec, total;
+    bool parts;  // ph twice more
 };
-WsLayout workspace_layout(const Geom& g, int kind);
+WsLayout workspace_layout(const Geom& g, int kind, size_t limit);  // limit in bytes; 0: none
 void workspace_carve(const Geom& g, const WsLayout& L, unsigned char* base, Workspace* w);
 cudaError_t run_forward(const Geom& g, const DeviceTables& t, const Workspace& w, const Scalars& s,
                         int kind, int m, const float* p0, float* f, cudaStream_t st, Profiler* prof);

@@ -59,7 +59,7 @@ struct ZKernels {
 ZKernels z_kernels_for(int nz);
 
 // Line passes of the time step (pat_line.cuh).
-enum LineMode { LM_STEP = 0, LM_INIT = 1, LM_FIN = 2 };
+enum LineMode { LM_STEP = 0, LM_INIT = 1, LM_FIN = 2, LM_RECORD = 3 };
 enum LineFlag {
     LF_NO_OLD1 = 1, LF_NO_OLD2 = 2, LF_ACCUM = 4, LF_RECORD = 8, LF_INJECT = 16,
     LF_LATE_WAIT = 32,    // wait for the predecessor only before fetching the spectrum added to
@@ -75,6 +75,8 @@ struct LineArgs {
     const float2* twi;          // per-thread twiddles of the inverse transform's first half, [k][r]
     const float2* twf;          // ... and of the forward transform's first half (LineKernels docs)
     const float2* in;           // 3D half spectrum read (LM_STEP, LM_INIT)
+    const float2* in2;          // two more parts of it, added in this order (NULL: none)
+    const float2* in3;
     float2* out;                // 3D half spectrum written or accumulated (LM_STEP, LM_FIN)
     float2* st1;                // mixed-representation states, tile-major [B][tile][L][TC]
     float2* st2;
@@ -117,6 +119,16 @@ struct LineKernels {
 };
 
 LineKernels line_kernels_for(int len);  // pass[] all NULL for a length without kernels
+
+// The three passes of a step in one launch (pat_step.cuh).
+struct StepArgs {
+    LineArgs a[3];  // by axis (z, y, x)
+    int first[2];   // first block of the z and y tiles; the x tiles are blocks 0 ..
+};
+typedef void (*StepKernel)(StepArgs);
+static constexpr int kStepThreads = 128;
+StepKernel step_kernel_r3();
+StepKernel step_kernel_r4();
 
 LineKernels line_kernels_l8();
 LineKernels line_kernels_l16();

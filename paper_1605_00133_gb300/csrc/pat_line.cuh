@@ -131,7 +131,12 @@ __device__ __forceinline__ float2 wr(int k) {
     return make_float2(w16c(k * (16 / R)), DIR * w16s(k * (16 / R)));
 }
 
-template <int L, int AX, bool STREAM>
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return cadd(a, b); }
+__device__ __forceinline__ float4 vadd(float4 a, float4 b) {
+    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+
+template <int L, int AX, bool STREAM, bool PARTS>
 struct LineCtx {
     using S = LS<L>;
     static constexpr int A = S::A, B = S::B, TC = S::TC, XN = S::XN;
@@ -156,7 +161,7 @@ struct LineCtx {
     int ka, kb;     // x lines: kz, ky
     int ma, mb;     // x lines: the mirror line's kz, ky
 
-    __device__ LineCtx(const LineArgs& args, float2* smem) : a(args) {
+    __device__ LineCtx(const LineArgs& args, float2* smem, int tile) : a(args) {
         buf0 = smem;
         buf1 = smem + S::BUF;
         pf1 = smem + 2 * S::BUF;
@@ -170,12 +175,12 @@ struct LineCtx {
         r = tid / TC;
         xr = PAIR ? (S::PNEW ? ((r & 1) | ((r >> 2) << 1)) : (r >> 1)) : r;
         xh = PAIR ? (S::PNEW ? ((r >> 1) & 1) : (r & 1)) : 0;
-        col0 = blockIdx.x * TC;
+        col0 = tile * TC;
         col = col0 + cl;
         vcol = col < a.ncols;
         xact = vcol && (PAIR || r < B);
         b = blockIdx.y;
-        tbase = ((size_t)b * gridDim.x + blockIdx.x) * (size_t)(L * TC);
+        tbase = ((size_t)b * (PARTS ? a.g.ntile[AX] : gridDim.x) + tile) * (size_t)(L * TC);
         pbase = (size_t)b * a.g.nspec;
         sgn = xh ? make_float2(-1.f, -1.f) : make_float2(1.f, 1.f);
         ti = a.twi + r;
@@ -305,17 +310,29 @@ struct LineCtx {
     }
 
     // ---- 3D spectrum access in the k-space layout
-    __device__ __forceinline__ void load_k(const float2* __restrict__ in, float2* v) const {
+    // element i of the spectrum read: with PARTS the sum of what the x, y and z passes wrote
+    template <class T>
+    __device__ __forceinline__ T ld_spec(size_t i) const {
+        const T v = __ldcg(reinterpret_cast<const T*>(a.in + pbase) + i);
+        if constexpr (PARTS) {
+            if (a.in2) {
+                const T p = __ldcg(reinterpret_cast<const T*>(a.in2 + pbase) + i);
+                const T q = __ldcg(reinterpret_cast<const T*>(a.in3 + pbase) + i);
+                return vadd(vadd(v, p), q);
+            }
+        }
+        return v;
+    }
+    __device__ __forceinline__ void load_k(float2* v) const {
         if (AX == 0) {
             if (vcol) {
 #pragma unroll
-                for (int k2 = 0; k2 < B; k2++) v[k2] = __ldcg(in + pbase + (size_t)(r + A * k2) * a.ncols + col);
+                for (int k2 = 0; k2 < B; k2++) v[k2] = ld_spec<float2>((size_t)(r + A * k2) * a.ncols + col);
             }
         } else if (AX == 1) {
             const int nrows = min(TC, a.ncols - col0);
-            const float4* blk = reinterpret_cast<const float4*>(in + pbase + (size_t)col0 * L);
             for (int e = threadIdx.x; e < nrows * (L / 2); e += S::NT) {
-                const float4 w = __ldcg(blk + e);
+                const float4 w = ld_spec<float4>((size_t)col0 * (L / 2) + e);
                 const int row = (2 * e) / L, pt = (2 * e) % L;
                 float2* d = buf1 + row * S::PITCH + pt;
                 d[0] = make_float2(w.x, w.y);
@@ -330,15 +347,35 @@ struct LineCtx {
             // bin j = r + A k2 with r < A: j <= L/2 exactly for k2 < B/2, and for k2 = B/2 when r = 0
             if (vcol) {
                 const int nxh = a.g.nxh, ny = a.g.ny;
-                const float2* own = in + pbase + (size_t)ka * nxh * ny + kb;
-                const float2* mir = in + pbase + (size_t)ma * nxh * ny + mb;
+                const size_t own = (size_t)ka * nxh * ny + kb, mir = (size_t)ma * nxh * ny + mb;
 #pragma unroll
                 for (int k2 = 0; k2 < B; k2++) {
                     const int j = r + A * k2;
-                    if (k2 < B / 2 || (k2 == B / 2 && r == 0)) v[k2] = __ldcg(own + (size_t)j * ny);
-                    else v[k2] = cconj(__ldcg(mir + (size_t)(L - j) * ny));
+                    if (k2 < B / 2 || (k2 == B / 2 && r == 0)) v[k2] = ld_spec<float2>(own + (size_t)j * ny);
+                    else v[k2] = cconj(ld_spec<float2>(mir + (size_t)(L - j) * ny));
                 }
             }
+        }
+    }
+    // plane spectrum at z = zs of the z lines' values v: (1/nz) sum_kz p^(kz) e^{+2 pi i kz zs / nz}; this
+    // thread's part, then (after a barrier) the sum over the A threads of the line, through xb
+    __device__ __forceinline__ void record_part(const float2* v, float2* xb) const {
+        float2 part = make_float2(0.f, 0.f);
+        if (vcol) {
+#pragma unroll
+            for (int k2 = 0; k2 < B; k2++) {
+                const int kz = r + A * k2;
+                part = cadd(part, cmul(v[k2], cconj(__ldg(a.tw + ((kz * a.zs) & (L - 1))))));
+            }
+        }
+        xb[r * TC + cl] = part;
+    }
+    __device__ __forceinline__ void record_sum(const float2* xb) const {
+        if (vcol && r == 0) {
+            float2 sum = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int rr = 0; rr < A; rr++) sum = cadd(sum, xb[rr * TC + cl]);
+            a.rec[(size_t)b * a.plane_bs + col] = cscale(sum, a.s_rec);
         }
     }
     // write (or add, LF_ACCUM) the k-space layout values to the 3D spectrum; z lines return the
@@ -432,6 +469,10 @@ struct LineCtx {
     // mbarrier; the barrier initialisation is published by a __syncthreads before any thread waits.
     __device__ __forceinline__ void issue_copies(bool old1, bool old2) const {
         if (threadIdx.x != 0) return;
+        issue_tables();
+        issue_states(old1, old2);
+    }
+    __device__ __forceinline__ void issue_tables() const {
         mbar_init(bar + 0, 1);
         mbar_init(bar + 1, 1);
         mbar_init(bar + 2, 1);
@@ -440,6 +481,8 @@ struct LineCtx {
             mbar_arrive_expect_tx(bar + 0, S::TAB_BYTES);
             bulk_copy_g2s(tab2, a.tabs, S::TAB_BYTES, bar + 0);
         }
+    }
+    __device__ __forceinline__ void issue_states(bool old1, bool old2) const {
         constexpr unsigned PART = S::TILE_BYTES / S::BULK_PARTS;
         constexpr int PART2 = (int)(PART / sizeof(float2));
         static_assert(PART % 16 == 0, "bulk copy pieces of 16-byte multiples");
@@ -535,21 +578,24 @@ struct LineCtx {
     }
 };
 
-template <int L, int AX, bool STREAM>
-__global__ void __launch_bounds__(LS<L>::NT, LS<L>::MINB) line_pass_kernel(LineArgs a) {
+// One pass over tile `tile` of the lines of axis AX.  PARTS: the passes of a step run side by side, each reading the
+// sum of what the three passes of the step before wrote and writing a spectrum of its own (LM_STEP, LM_RECORD only).
+template <int L, int AX, bool STREAM, bool PARTS>
+__device__ __forceinline__ void line_pass(const LineArgs& a, int tile) {
     using S = LS<L>;
     constexpr int A = S::A, B = S::B;
+    if (PARTS && AX != 0 && a.mode == LM_RECORD) return;
     extern __shared__ float4 smem_raw[];
-    LineCtx<L, AX, STREAM> c(a, reinterpret_cast<float2*>(smem_raw));
-    const bool late = (a.flags & LF_LATE_WAIT) != 0;
-    if (!late) pdl_wait();
-    if (!(a.flags & (LF_TRIGGER_MID | LF_TRIGGER_END))) pdl_trigger();
+    LineCtx<L, AX, STREAM, PARTS> c(a, reinterpret_cast<float2*>(smem_raw), tile);
+    const bool late = !PARTS && (a.flags & LF_LATE_WAIT) != 0;
+    if (!PARTS && !late) pdl_wait();
+    if (!PARTS && !(a.flags & (LF_TRIGGER_MID | LF_TRIGGER_END))) pdl_trigger();
     constexpr int XN = S::XN;
     float2 v[B];
     float2 x[XN];
-    const bool accum = (a.flags & LF_ACCUM) != 0;
+    const bool accum = !PARTS && (a.flags & LF_ACCUM) != 0;
 
-    if (a.mode == LM_FIN) {
+    if (!PARTS && a.mode == LM_FIN) {
         // adjoint image term: out += F_i (c1[0] st1)
 #pragma unroll
         for (int q = 0; q < XN; q++) {
@@ -567,18 +613,43 @@ __global__ void __launch_bounds__(LS<L>::NT, LS<L>::MINB) line_pass_kernel(LineA
     const float* c2[3] = {a.c2[0], a.c2[1], a.c2[2]};
     const bool old1 = (a.flags & LF_NO_OLD1) == 0, old2 = (a.flags & LF_NO_OLD2) == 0;
     if (a.mode == LM_STEP) {
-        c.issue_copies(old1, old2);
-        if (!S::BULK) {
-            c.prefetch(a.st1, c.pf1, old1);
-            c.prefetch(a.st2, c.pf2, old2);
+        if (PARTS) {
+            if (threadIdx.x == 0) c.issue_tables();
+        } else {
+            c.issue_copies(old1, old2);
+            if (!S::BULK) {
+                c.prefetch(a.st1, c.pf1, old1);
+                c.prefetch(a.st2, c.pf2, old2);
+            }
         }
         if (S::STAGE) c.stage(dk, c1, c2);
-        const float* kp = a.kap + (size_t)blockIdx.x * (L * S::TC) + c.r * S::TC + c.cl;
+        const float* kp = a.kap + (size_t)tile * (L * S::TC) + c.r * S::TC + c.cl;
 #pragma unroll
         for (int k2 = 0; k2 < B; k2++) kap[k2] = c.vcol ? ldg_stream(kp + k2 * A * S::TC) : 0.f;
     }
-    c.load_k(a.in, v);
-    if (a.mode == LM_INIT) {
+    if (PARTS) {
+        pdl_wait();     // tables and kappa are constant; everything else is the step before's
+        pdl_trigger();
+        if (a.mode == LM_STEP) {
+            if (threadIdx.x == 0) c.issue_states(old1, old2);
+            if (!S::BULK) {
+                c.prefetch(a.st1, c.pf1, old1);
+                c.prefetch(a.st2, c.pf2, old2);
+            }
+        }
+    }
+    c.load_k(v);
+    const bool record = AX == 0 && (a.flags & LF_RECORD) != 0;
+    if (PARTS && record) {
+        // the plane of the step before, whose parts are complete only now
+        c.record_part(v, c.buf1);
+        if (a.mode == LM_RECORD) {
+            __syncthreads();
+            c.record_sum(c.buf1);
+            return;
+        }
+    }
+    if (!PARTS && a.mode == LM_INIT) {
         // forward start: st2 = F_i^-1[p^] s_pre  (rho_i^0 = p0 / (3 c^2))
         c.factor(v, nullptr, nullptr, a.s_pre);
         c.inv(v, x, c.buf0);
@@ -589,7 +660,8 @@ __global__ void __launch_bounds__(LS<L>::NT, LS<L>::MINB) line_pass_kernel(LineA
         return;
     }
 
-    __syncthreads();  // publishes the mbarrier initialisation
+    __syncthreads();  // publishes the mbarrier initialisation (and the parts of the record)
+    if (PARTS && record) c.record_sum(c.buf1);
     const bool ok0 = S::STAGE ? c.wait_copy(0) : true;  // the tables
     c.factor(v, dk[0], kap, a.s_pre);
     if (!S::BULK) cp_async_wait<1>();  // state 1 has landed; the barrier inside inv() publishes it
@@ -628,26 +700,16 @@ __global__ void __launch_bounds__(LS<L>::NT, LS<L>::MINB) line_pass_kernel(LineA
     }
     c.store_k(a.out, v, accum, pre);
 
-    if (AX == 0 && (a.flags & LF_RECORD)) {
-        // plane spectrum at z = zs: (1/nz) sum_kz p^(kz) e^{+2 pi i kz zs / nz}; partial sums over
-        // this thread's kz, then over the A threads of the line (buf0 is free, see store_k)
-        float2 part = make_float2(0.f, 0.f);
-        if (c.vcol) {
-#pragma unroll
-            for (int k2 = 0; k2 < B; k2++) {
-                const int kz = c.r + A * k2;
-                part = cadd(part, cmul(v[k2], cconj(__ldg(a.tw + ((kz * a.zs) & (L - 1))))));
-            }
-        }
-        c.buf0[c.r * S::TC + c.cl] = part;
+    if (!PARTS && record) {
+        c.record_part(v, c.buf0);  // buf0 is free, see store_k
         __syncthreads();
-        if (c.vcol && c.r == 0) {
-            float2 sum = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int rr = 0; rr < A; rr++) sum = cadd(sum, c.buf0[rr * S::TC + c.cl]);
-            a.rec[(size_t)c.b * a.plane_bs + c.col] = cscale(sum, a.s_rec);
-        }
+        c.record_sum(c.buf0);
     }
+}
+
+template <int L, int AX, bool STREAM>
+__global__ void __launch_bounds__(LS<L>::NT, LS<L>::MINB) line_pass_kernel(LineArgs a) {
+    line_pass<L, AX, STREAM, false>(a, blockIdx.x);
 }
 
 template <int L>

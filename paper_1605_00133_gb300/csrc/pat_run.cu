@@ -57,6 +57,7 @@ int plane_cluster_size(int nx, int ny) { return plane_kernels_for(nx, ny).cs; }
 static const char* g_config_what = "";
 const char* configure_failure() { return g_config_what; }
 
+static cudaError_t configure_step();
 cudaError_t configure_kernels(const Geom& g, int kind) {
     PlaneKernels pk = plane_kernels_for(g.nx, g.ny);
     ZKernels zk = z_kernels_for(g.nz);
@@ -78,15 +79,16 @@ cudaError_t configure_kernels(const Geom& g, int kind) {
     PAT_CFG(cudaFuncSetAttribute(zk.inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)zk.smem), "zfft_inv smem");
     for (int ax = 0; ax < 3; ax++) {
         LineKernels lk = line_kernels_for(g.len[ax]);
-        for (int stream = 0; stream < 2; stream++) {
-            if (!lk.pass[stream][ax]) {
+        for (const auto& form : lk.pass) {
+            if (!form[ax]) {
                 g_config_what = "no line kernel for this axis length";
                 return cudaErrorInvalidValue;
             }
-            PAT_CFG(cudaFuncSetAttribute(lk.pass[stream][ax], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lk.smem),
+            PAT_CFG(cudaFuncSetAttribute(form[ax], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lk.smem),
                     "line pass smem");
         }
     }
+    PAT_CFG(configure_step(), "step smem");
     PAT_CFG(configure_sampling(g, kind), "sampling smem");
 #undef PAT_CFG
     g_config_what = "";
@@ -208,6 +210,58 @@ cudaError_t launch_spread_plane(const Geom& g, const float2* tw_z, const float2*
     return cudaGetLastError();
 }
 
+// Which grids do a step in one launch (pat_step.cuh), by their tiles (CTAs), and in which form.  Loops of 64 steps,
+// three launches a step / one launch of the form for three / for four CTAs an SM:
+//   102 tiles (32^3) 569 / 291 / 291 us, 396 (64^3) 758 / 501 / 545, 534 (16x128x128) 827 / 556 / 610,
+//   788 (128x64x64) 1051 / 980 / 1012, 938 (16x256x128) 1003 / 914 / 913,
+//   1052 (32x128x128) 944 / 966 / 818, 1188 (three volumes of 64^3) 1037 / 1130 / 967,
+//   1584 (four volumes of 64^3) 1109 / - / 1293, 1602 (three of 16x128x128) 1161 / - / 1210.
+// So two rounds of CTAs over the SMs, 2 x 152 x 3 and 2 x 152 x 4: beyond that the passes fill the chip by themselves,
+// and the three spectra read instead of one cost more than the waits.
+int step_residency(const Geom& g) {
+    long long n = 0;
+    for (int ax = 0; ax < 3; ax++) n += (long long)g.ntile[ax] * g.B;
+    return n <= 2 * 152 * 3 ? 3 : n <= 2 * 152 * 4 ? 4 : 0;
+}
+
+static size_t step_smem(const Geom& g) {
+    size_t n = 0;
+    for (int ax = 0; ax < 3; ax++) n = std::max(n, line_kernels_for(g.len[ax]).smem);
+    return n;
+}
+
+static cudaError_t configure_step() {
+    // the kernels serve every grid: the most that any of them needs
+    size_t n = 0;
+    for (int len = 8; len <= 256; len *= 2) n = std::max(n, line_kernels_for(len).smem);
+    const cudaError_t e = cudaFuncSetAttribute(step_kernel_r3(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(step_kernel_r4(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
+}
+
+static cudaError_t launch_step(StepArgs& s, cudaStream_t st) {
+    const Geom& g = s.a[0].g;
+    s.first[1] = g.ntile[AX];
+    s.first[0] = g.ntile[AX] + g.ntile[AY];
+    return launch_pdl(step_residency(g) == 3 ? step_kernel_r3() : step_kernel_r4(),
+                      dim3((unsigned)(s.first[0] + g.ntile[AZ]), (unsigned)g.B), kStepThreads, step_smem(g), st, s);
+}
+
+// A pass of such a step: the spectrum read is in parts but for the first step's, and each pass writes one.
+static void set_parts(LineArgs& a, const Workspace& w, int ax, int cur, bool first) {
+    a.in = w.ph[cur];
+    a.in2 = first ? nullptr : w.part[cur][0];
+    a.in3 = first ? nullptr : w.part[cur][1];
+    a.out = ax == AX ? w.ph[cur ^ 1] : w.part[cur ^ 1][ax == AY ? 0 : 1];
+}
+
+// ph += y part + z part, in the order in which the passes add them
+__global__ void sum_parts_kernel(float2* __restrict__ ph, const float2* __restrict__ y, const float2* __restrict__ z,
+                                 long long n) {
+    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += gridDim.x * 256LL)
+        ph[i] = cadd(cadd(ph[i], y[i]), z[i]);
+}
+
 static LineArgs line_base(const Geom& g, const DeviceTables& t, const Workspace& w, int ax) {
     LineArgs a = {};
     a.g = g;
@@ -254,6 +308,7 @@ cudaError_t run_forward(const Geom& g, const DeviceTables& t, const Workspace& w
     const ZKernels zk = z_kernels_for(g.nz);
     if (!pk.rfft || !zk.fwd) return cudaErrorInvalidValue;
     float* rec = (kind == PAT_SAMPLE_FULL) ? f : w.rec;
+    const bool parts = w.part[0][0] != nullptr;
     const long long M = g.m_plane;
 
     // p^0 = F p0; the record's plane 0 is p0's detection plane, taken through its (kx, ky) spectrum
@@ -295,7 +350,23 @@ cudaError_t run_forward(const Geom& g, const DeviceTables& t, const Workspace& w
             la[ax].s_post = (float)c2;
         }
         const NvtxRange loop("forward time loop");
-        for (int n = 0; n + 1 < g.T; n++) {
+        if (parts) {
+            // a step records the plane that it reads; one more launch records the last
+            StepArgs sa;
+            for (int ax = 0; ax < 3; ax++) sa.a[ax] = la[ax];
+            for (int n = 0; n < g.T; n++) {
+                for (int ax = 0; ax < 3; ax++) {
+                    LineArgs& a = sa.a[ax];
+                    set_parts(a, w, ax, n & 1, n == 0);
+                    set_pass_tables(a, t, ax, (n == 0) ? PS_FWD0 : PS_FWD);
+                    a.flags = (n == 0 ? LF_NO_OLD1 : 0) | (ax == AZ && n > 0 ? LF_RECORD : 0);
+                    a.rec = w.rk + (size_t)n * g.nplane;
+                    if (n + 1 == g.T) a.mode = LM_RECORD;
+                }
+                PAT_TRY(timed(prof, KC_STEP, st, [&] { return launch_step(sa, st); }));
+            }
+        }
+        for (int n = 0; !parts && n + 1 < g.T; n++) {
             float2* cur = w.ph[n & 1];
             float2* nxt = w.ph[(n + 1) & 1];
             for (int ax : kPassOrder) {
@@ -352,6 +423,7 @@ cudaError_t run_adjoint(const Geom& g, const DeviceTables& t, const Workspace& w
     const long long s_bs = (long long)g.T * g.nplane;
     PAT_TRY(launch_spread_plane(g, t.tw[AZ], w.rk + (size_t)(g.T - 1) * g.nplane, s_bs, w.ph[0], st));
 
+    const bool parts = w.part[0][0] != nullptr;
     LineArgs la[3];
     for (int ax = 0; ax < 3; ax++) {
         la[ax] = line_base(g, t, w, ax);
@@ -362,7 +434,25 @@ cudaError_t run_adjoint(const Geom& g, const DeviceTables& t, const Workspace& w
     }
     int cur = 0;
     const NvtxRange loop("adjoint time loop");
-    for (int n = g.T - 2; n >= 0; n--) {
+    if (parts) {
+        StepArgs sa;
+        for (int ax = 0; ax < 3; ax++) sa.a[ax] = la[ax];
+        for (int n = g.T - 2; n >= 0; n--, cur ^= 1) {
+            for (int ax = 0; ax < 3; ax++) {
+                LineArgs& a = sa.a[ax];
+                set_parts(a, w, ax, cur, n == g.T - 2);
+                set_pass_tables(a, t, ax, (n == 0) ? PS_ADJ0 : PS_ADJ);
+                a.flags = (n == g.T - 2 ? (LF_NO_OLD1 | LF_NO_OLD2) : 0) | (ax == AZ ? LF_INJECT : 0);
+                a.inj = w.rk + (size_t)n * g.nplane;
+            }
+            PAT_TRY(timed(prof, KC_STEP, st, [&] { return launch_step(sa, st); }));
+        }
+        const long long n = (long long)g.B * g.nspec;
+        sum_parts_kernel<<<(unsigned)std::min<long long>((n + 255) / 256, 4096), 256, 0, st>>>(w.ph[cur], w.part[cur][0],
+                                                                                             w.part[cur][1], n);
+        PAT_TRY(cudaGetLastError());
+    }
+    for (int n = g.T - 2; !parts && n >= 0; n--) {
         for (int ax : kPassOrder) {
             LineArgs& a = la[ax];
             a.in = w.ph[cur];
