@@ -172,8 +172,8 @@ struct SolverWs {
     float* q2 = nullptr;                                                            // prox: N
     float *ax = nullptr, *axp = nullptr, *ay = nullptr, *r = nullptr;              // data, T*m
     double *gdat = nullptr, *bdat = nullptr;                                        // data, FP64
-    double *partial = nullptr, *result = nullptr;                                   // reductions
-    double* host = nullptr;                                                         // pinned
+    double* partial = nullptr;                                                      // reductions
+    double* host = nullptr;                                                         // pinned: their results
 };
 
 }  // namespace pat

@@ -485,10 +485,22 @@ __device__ __forceinline__ double red_term(const RedArgs& r, size_t i) {
     }
 }
 
-__global__ void reduce_stage1_kernel(RedArgs r, double* __restrict__ partial) {
+// Up to kRedMost sums at once, one per blockIdx.y (stage 1) or block (stage 2), and one wait of the host for them
+// all: what an iteration needs (data term, TV, change) took three pairs of launches, copies and waits, during each of
+// which the GPU stood still for about 20 us.  Stage 2 writes the results to pinned host memory itself.
+constexpr int kRedMost = 3;
+struct RedSet {
+    RedArgs r[kRedMost];
+    int nb[kRedMost];  // blocks of each sum
+};
+
+__global__ void reduce_stage1_kernel(const __grid_constant__ RedSet s, double* partial) {
     __shared__ double sh[kRedThreads / 32];
+    const RedArgs& r = s.r[blockIdx.y];
+    const int nb = s.nb[blockIdx.y];
+    if ((int)blockIdx.x >= nb) return;
     double acc = 0.0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < r.n; i += (size_t)gridDim.x * blockDim.x)
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < r.n; i += (size_t)nb * blockDim.x)
         acc += red_term(r, i);
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
@@ -496,21 +508,23 @@ __global__ void reduce_stage1_kernel(RedArgs r, double* __restrict__ partial) {
     if (threadIdx.x == 0) {
         double t = 0.0;
         for (int w = 0; w < kRedThreads / 32; w++) t += sh[w];
-        partial[blockIdx.x] = t;
+        partial[blockIdx.y * kRedBlocks + blockIdx.x] = t;
     }
 }
 
-__global__ void reduce_stage2_kernel(const double* __restrict__ partial, int np, double* __restrict__ out) {
+__global__ void reduce_stage2_kernel(const __grid_constant__ RedSet s, const double* partial, double* out) {
     __shared__ double sh[kRedThreads];
+    const double* p = partial + blockIdx.x * kRedBlocks;
+    const int np = s.nb[blockIdx.x];
     double acc = 0.0;
-    for (int i = threadIdx.x; i < np; i += blockDim.x) acc += partial[i];
+    for (int i = threadIdx.x; i < np; i += blockDim.x) acc += p[i];
     sh[threadIdx.x] = acc;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
+    for (int h = blockDim.x / 2; h > 0; h >>= 1) {
+        if ((int)threadIdx.x < h) sh[threadIdx.x] += sh[threadIdx.x + h];
         __syncthreads();
     }
-    if (threadIdx.x == 0) *out = sh[0];
+    if (threadIdx.x == 0) out[blockIdx.x] = sh[0];
 }
 
 // ------------------------------------------------------------------------------ host helpers
@@ -523,15 +537,21 @@ struct Ctx {
     TvDims td;
 };
 
-static pat_status reduce(Ctx& c, const RedArgs& r, double* out) {
+// n sums; the host waits for them
+static pat_status reduce(Ctx& c, const RedArgs* r, int n, double* out) {
     SolverWs& w = c.G->sw;
-    const int nb = (int)std::min<size_t>(kRedBlocks, std::max<size_t>(1, (r.n + kRedThreads - 1) / kRedThreads));
-    reduce_stage1_kernel<<<nb, kRedThreads, 0, c.st>>>(r, w.partial);
-    reduce_stage2_kernel<<<1, kRedThreads, 0, c.st>>>(w.partial, nb, w.result);
+    RedSet s = {};
+    int most = 1;
+    for (int k = 0; k < n; k++) {
+        s.r[k] = r[k];
+        s.nb[k] = (int)std::min<size_t>(kRedBlocks, std::max<size_t>(1, (r[k].n + kRedThreads - 1) / kRedThreads));
+        most = std::max(most, s.nb[k]);
+    }
+    reduce_stage1_kernel<<<dim3((unsigned)most, (unsigned)n), kRedThreads, 0, c.st>>>(s, w.partial);
+    reduce_stage2_kernel<<<n, kRedThreads, 0, c.st>>>(s, w.partial, w.host);
     PAT_CUDA(cudaGetLastError(), "reduction launch");
-    PAT_CUDA(cudaMemcpyAsync(w.host, w.result, sizeof(double), cudaMemcpyDeviceToHost, c.st), "reduction copy");
     PAT_CUDA(cudaStreamSynchronize(c.st), "reduction sync");
-    *out = w.host[0];
+    for (int k = 0; k < n; k++) out[k] = w.host[k];
     return PAT_OK;
 }
 
@@ -547,8 +567,7 @@ static pat_status ensure_ws(pat_grid* G, bool solver) {
         if (st == PAT_OK) st = grid_alloc(G, (void**)&w.xi2, 3 * N * sizeof(float), "prox dual");
         if (st == PAT_OK) st = grid_alloc(G, (void**)&w.z, N * sizeof(float), "prox input copy");
         if (st == PAT_OK) st = grid_alloc(G, (void**)&w.q2, N * sizeof(float), "prox iterate");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.partial, kRedBlocks * sizeof(double), "reduction");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.result, sizeof(double), "reduction");
+        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.partial, kRedMost * kRedBlocks * sizeof(double), "reduction");
         if (st == PAT_OK) {
             cudaError_t e = cudaMallocHost((void**)&w.host, 4 * sizeof(double));
             if (e != cudaSuccess) return set_cuda_error(e, "cudaMallocHost(reduction)");
@@ -705,22 +724,26 @@ static pat_status tv_prox_run(Ctx& c, const float* p, float* q, double alpha, in
     return PAT_OK;
 }
 
-static pat_status energy(Ctx& c, const float* ax, const float* x, double lam, double* E) {
-    RedArgs r = {};
-    r.op = RED_SUMSQ_DIFF;
-    r.a = ax;
-    r.gd = c.G->sw.gdat;
-    r.n = c.D;
-    double dfit = 0.0, tvv = 0.0;
-    pat_status st = reduce(c, r, &dfit);
+// E = 1/2 ||ax - g||^2 + lam TV(x) and, with xp, change = ||x - xp||_1
+static pat_status energy(Ctx& c, const float* ax, const float* x, double lam, double* E, const float* xp, double* change) {
+    RedArgs r[kRedMost] = {};
+    r[0].op = RED_SUMSQ_DIFF;
+    r[0].a = ax;
+    r[0].gd = c.G->sw.gdat;
+    r[0].n = c.D;
+    r[1].op = RED_TV;
+    r[1].a = x;
+    r[1].n = c.N;
+    r[1].d = c.td;
+    r[2].op = RED_ABS_DIFF;
+    r[2].a = x;
+    r[2].b = xp;
+    r[2].n = c.N;
+    double v[kRedMost] = {};
+    const pat_status st = reduce(c, r, xp ? 3 : 2, v);
     if (st != PAT_OK) return st;
-    RedArgs t = {};
-    t.op = RED_TV;
-    t.a = x;
-    t.n = c.N;
-    t.d = c.td;
-    if ((st = reduce(c, t, &tvv)) != PAT_OK) return st;
-    *E = 0.5 * dfit + lam * tvv;
+    *E = 0.5 * v[0] + lam * v[1];
+    if (xp) *change = v[2];
     return PAT_OK;
 }
 
@@ -778,7 +801,7 @@ static pat_status power_iteration(Ctx& c, int iters, uint64_t seed, double* L) {
     r.op = RED_SUMSQ;
     r.a = w.x;
     r.n = c.N;
-    pat_status st = reduce(c, r, &nrm);
+    pat_status st = reduce(c, &r, 1, &nrm);
     if (st != PAT_OK) return st;
     nrm = sqrt(nrm);
     double lam = 0.0;
@@ -788,7 +811,7 @@ static pat_status power_iteration(Ctx& c, int iters, uint64_t seed, double* L) {
         if ((st = A_fwd(c, w.x, w.ax)) != PAT_OK) return st;
         if ((st = A_adj(c, w.ax, w.x)) != PAT_OK) return st;
         r.a = w.x;
-        if ((st = reduce(c, r, &nrm)) != PAT_OK) return st;
+        if ((st = reduce(c, &r, 1, &nrm)) != PAT_OK) return st;
         nrm = sqrt(nrm);
         lam = nrm;
         if (!(nrm > 0)) break;
@@ -812,7 +835,7 @@ static pat_status fista(Ctx& c, const pat_solve_params& P, double eta, FistaOut*
     pat_status st;
     if ((st = A_fwd(c, xp, axp)) != PAT_OK) return st;
     double Ep = 0.0;
-    if ((st = energy(c, axp, xp, P.lambda, &Ep)) != PAT_OK) return st;
+    if ((st = energy(c, axp, xp, P.lambda, &Ep, nullptr, nullptr)) != PAT_OK) return st;
     PAT_CUDA(cudaMemcpyAsync(y, xp, c.N * sizeof(float), cudaMemcpyDeviceToDevice, c.st), "fista init");
     PAT_CUDA(cudaMemcpyAsync(ay, axp, c.D * sizeof(float), cudaMemcpyDeviceToDevice, c.st), "fista init");
     double t = 1.0, best = Ep;
@@ -821,8 +844,8 @@ static pat_status fista(Ctx& c, const pat_solve_params& P, double eta, FistaOut*
         if ((st = gradient(c, ay, w.grad)) != PAT_OK) return st;
         if ((st = prox_step(c, y, w.grad, eta, P.lambda, P.prox_iters, x)) != PAT_OK) return st;
         if ((st = A_fwd(c, x, ax)) != PAT_OK) return st;
-        double E = 0.0;
-        if ((st = energy(c, ax, x, P.lambda, &E)) != PAT_OK) return st;
+        double E = 0.0, change = 0.0;
+        if ((st = energy(c, ax, x, P.lambda, &E, xp, &change)) != PAT_OK) return st;
         if (E > Ep) {
             out->restarts++;
             t = 1.0;
@@ -831,7 +854,7 @@ static pat_status fista(Ctx& c, const pat_solve_params& P, double eta, FistaOut*
             for (int b = 0; b <= P.max_backtrack; b++) {
                 if ((st = prox_step(c, xp, w.grad, eta_b, P.lambda, P.prox_iters, x)) != PAT_OK) return st;
                 if ((st = A_fwd(c, x, ax)) != PAT_OK) return st;
-                if ((st = energy(c, ax, x, P.lambda, &E)) != PAT_OK) return st;
+                if ((st = energy(c, ax, x, P.lambda, &E, xp, &change)) != PAT_OK) return st;
                 if (E <= Ep) break;
                 eta_b *= 0.5;
             }
@@ -839,16 +862,10 @@ static pat_status fista(Ctx& c, const pat_solve_params& P, double eta, FistaOut*
                 PAT_CUDA(cudaMemcpyAsync(x, xp, c.N * sizeof(float), cudaMemcpyDeviceToDevice, c.st), "fista keep");
                 PAT_CUDA(cudaMemcpyAsync(ax, axp, c.D * sizeof(float), cudaMemcpyDeviceToDevice, c.st), "fista keep");
                 E = Ep;
+                change = 0.0;
             }
         }
         out->iterations++;
-        double change = 0.0;
-        RedArgs r = {};
-        r.op = RED_ABS_DIFF;
-        r.a = x;
-        r.b = xp;
-        r.n = c.N;
-        if ((st = reduce(c, r, &change)) != PAT_OK) return st;
         const double t_next = 0.5 * (1.0 + sqrt(1.0 + 4.0 * t * t));
         const double beta = (t - 1.0) / t_next;
         axpby_kernel<<<ew_blocks(c.N), 256, 0, c.st>>>(y, x, xp, (float)(1.0 + beta), (float)-beta, c.N);
@@ -977,7 +994,7 @@ extern "C" pat_status pat_bregman_solve(pat_grid* G, const float* f, const float
         q.a = w.axp;
         q.b = f;
         q.n = c.D;
-        if ((st = reduce(c, q, &res2)) != PAT_OK) return st;
+        if ((st = reduce(c, &q, 1, &res2)) != PAT_OK) return st;
         const double res = sqrt(res2);
         if (k < 64) rep.residual[k] = res;
         rep.n_residual = std::min(k + 1, 64);
