@@ -9,8 +9,8 @@
 //   the TMA unit: one box row (one voxel's channels, up to 64 bytes; 128 bytes in 1.2 cycles) per cycle and
 //     SM, whatever the row's width: so a row of 48 (or 96, ...) channels is fetched as one (two) rows of 64
 //     channels, the missing ones zero-filled, not in 16-channel pieces.
-// conv3_ring_kernel (few channels, large volumes) fetches every line a few times and is bound by its MMAs;
-// conv3_tc_kernel serves every other shape, one shifted box per tap.
+// conv3_ring_kernel (few channels, large volumes) fetches every line a few times and serves three taps with one
+// MMA; conv3_tc_kernel serves every other shape, one shifted box per tap.
 // conv3_tc_kernel: a CTA owns one tile of M = 128 voxels, a bx x by x bz box of the volume (x fastest), and
 // BN output channels.  One K step is one tap and CK input channels:
 //   A: the voxel box shifted by the tap, loaded by a 4D tensor map over (channel, x, y, z); parts of
@@ -160,6 +160,16 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float* v) {
 #pragma unroll
     for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
 }
+
+// zeros into 16 consecutive FP32 columns of this thread's tensor-memory lane (tc_wait_st() before they are relied on)
+__device__ __forceinline__ void tc_zero16(uint32_t taddr) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(
+            taddr),
+        "r"(0u)
+        : "memory");
+}
+__device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // Rounds 16 channels of a voxel to BF16 and stores them.  With a mask (the activation a gradient is taken
 // through) channels where it is not positive are stored as zero.
@@ -351,25 +361,30 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(const __grid_cons
 // ---------------------------------------------------------------------------------------------
 // The same convolution for few channels on large volumes (lines up to 128 voxels, weights that fit shared
 // memory): a persistent kernel.  A CTA keeps its weights in shared memory and walks along z through a
-// column of one M tile (by lines of W voxels), holding a ring of input planes of by + 2 lines; steps
+// column of one M tile (by lines of W voxels), with a ring of input planes of by + 2 lines; steps
 // (column, z) are numbered column by column and each CTA takes an equal contiguous range.  A tap's operand
-// is 128 rows of a plane from another start: dz planes, dy lines and dx voxels on.
+// is 128 rows of a plane from another start: dy lines and dx voxels on.
 //   Lines over 64 voxels (by = 1): a plane's lines are W + 2 voxels (x = -1 .. W), in parts of 16 channels
 //     (32-byte rows), up to four; the operand starts dy (W + 2) + dx rows on.  The 32-byte swizzle is applied
 //     to shared-memory address bits by the TMA unit and the tensor core alike, so any row may be the first.
 //   Shorter lines (16 or 32 channels): every plane is held three times, shifted by dx, its lines bx voxels (W
 //     rounded up to 8), so that operands start at multiples of 8 rows and by lines fill the 128 rows.
-// Per tile the MMAs, 27 per 16 channels, are what is left: 27 x 46 = 1242 cycles at 16 channels, beside 390
-// rows (cycles) of the TMA unit; the epilogue works on a ring of accumulators, two groups of four warps
-// taking alternate tiles.  64x128x128 voxels: 16 -> 16 channels 137 -> 50 us, 48 -> 16 371 -> 114 us,
-// 16 -> 48 379 -> 54 us (one box per tap, and MMAs issued from one lane, before).
+// A plane enters three outputs, z + 1, z and z - 1, through the taps dz = -1, 0, 1.  Their accumulators lie side by
+// side in a ring of tensor-memory columns, and the three dz of a (dy, dx) in the weights, so one MMA of 3 bn columns
+// serves all three: 9 MMAs a plane of 16 channels instead of 27 of a third the width, which take no less (see
+// above).  An output still sums its taps in order: all of plane z - 1, then z, then z + 1.  Since one instruction
+// covers outputs that begin and outputs that go on, the epilogue leaves zeros in the accumulators it has read.
+// The epilogue is two groups of four warps taking alternate outputs.  64x128x128 voxels, one box per tap and MMAs
+// issued from one lane -> 27 MMAs -> 9 MMAs: 16 -> 16 channels 137 -> 50 -> 30 us, 48 -> 16 371 -> 114 -> 59, 16 -> 48
+// 379 -> 54 -> 44.  What bounds it now: per plane about 60 cycles an MMA and 350 of waits and issue (16 -> 16; the TMA
+// unit alone takes 21 us), the MMAs (48 -> 16), the epilogue's stores (16 -> 48: 37 us without).
 // Other shapes use the kernel above: longer lines, more channels (weights and planes do not fit, and its K
 // steps are bound less by the TMA unit), and volumes of less than four tiles an SM (the weights would be
 // fetched for too little work).
 // ---------------------------------------------------------------------------------------------
 
 constexpr int kRingThreads = 320;  // producer, MMA issuer, 2 x 4 epilogue warps
-constexpr int kMaxPlanes = 8, kMaxAcc = 8;
+constexpr int kMaxPlanes = 8, kMaxAcc = 16;
 
 struct ConvRingArgs {
     __nv_bfloat16* y;
@@ -381,7 +396,7 @@ struct ConvRingArgs {
     int ncopies;              // copies of a plane shifted by dx (1: the lines have a halo), from x = -1
     int steps_per_cta, steps; // (column, z) steps
     int relu;
-    int nplanes, nacc, acc_cols;
+    int nplanes, nacc;        // ring of input planes, of accumulators (bn columns each)
     uint32_t box_bytes;       // one part of one copy of a plane
     uint32_t dxstep;          // from tap dx to dx + 1, in 16-byte units: a copy or a row
 };
@@ -432,7 +447,10 @@ __global__ void __launch_bounds__(kRingThreads, 1)
     if (warp == 0 && lane == 0) {
         // producer: the weights, then the planes z-1 .. z+1 of every step in order, each once per run of z
         mbar_arrive_expect_tx(&wfull, 27u * NP * a.bn * RB);
-        for (int q = 0; q < NP; q++) tma_load_3d(wts + q * 27 * a.bn * RB, &tmw, q * CK, n0, 0, &wfull);
+        // the weights of (dy, dx): those of dz = 1, 0, -1 behind one another
+        for (int q = 0; q < NP; q++)
+            for (int t = 0; t < 27; t++)
+                tma_load_3d(wts + ((q * 9 + t % 9) * 3 + 2 - t / 9) * a.bn * RB, &tmw, q * CK, n0, t, &wfull);
         const uint32_t tx_bytes = (uint32_t)(a.ncopies * NP * a.pitch * a.lines) * RB;
         int p = 0, slot = 0;
         uint32_t phase = 1;  // a fresh empty barrier's preceding phase counts as complete
@@ -463,58 +481,57 @@ __global__ void __launch_bounds__(kRingThreads, 1)
     } else if (warp == 1) {
         // MMA issuer (all lanes run the loop, one issues)
         const bool leader = elect_one();
-        const uint32_t idesc = mma_idesc(a.bn);
         const uint64_t da = kmajor_desc(smem_addr(planes), RB), db = kmajor_desc(smem_addr(wts), RB);
         const uint32_t hi = hi32(da);
         // address steps in 16-byte units: a plane, a part, dx, a line, one tap's weights, a part's
         const uint32_t pstep = plane_bytes >> 4, qstep = a.box_bytes >> 4, dxstep = a.dxstep;
         const uint32_t lstep = a.pitch * (RB / 16), wstep = a.bn * (RB / 16), wqstep = 27 * wstep;
+        // the nine (dy, dx) of the plane at x for n outputs, from accumulator acc and weight block b on
+        auto plane_mmas = [&](uint32_t x0, int acc, int b, int n) {
+            const uint32_t td = tmem + acc * a.bn, idesc = mma_idesc(n * a.bn), w0 = lo32(db) + b * wstep;
+#pragma unroll
+            for (int r = 0; r < 9; r++) {
+                const uint32_t x = x0 + (r % 3) * dxstep + (r / 3) * lstep, w = w0 + r * 3 * wstep;
+#pragma unroll
+                for (int q = 0; q < NP; q++) {
+                    tc_mma(td, x + q * qstep, hi, w + q * wqstep, hi, idesc, 1u);
+                    if (CK == 32) tc_mma(td, x + 2, hi, w + 2, hi, idesc, 1u);
+                }
+            }
+        };
         bool ok = mbar_wait(&wfull, 0, kPolls);
-        int slot = 0, acc = 0;      // ring slot of the next plane to wait for, accumulator
-        uint32_t pphase = 0, acc_phase = 1;
-        int first = 0;              // ring slot of plane z - 1 of the current step
+        int slot = 0, acc = 0;  // ring slots of the plane and of its first output
+        uint32_t pphase = 0, acc_phase = 0;
+        int fresh = 0;          // accumulator of the next output to begin
         for (int u = u0; u < u1 && ok;) {
             const int col = u / a.D, z0 = u - col * a.D, n = min(u1 - u, a.D - z0);
-            for (int i = 0; i < n; i++) {
-                for (int k = (i == 0) ? 3 : 1; k > 0 && ok; k--) {
-                    ok = mbar_wait(pfull + slot, pphase, kPolls);
-                    if (++slot == a.nplanes) {
-                        slot = 0;
-                        pphase ^= 1;
+            for (int i = -1; i <= n; i++) {
+                // plane z0 + i: outputs i - 1 .. i + 1 of this run, of which i + 1 begins and i - 1 is complete
+                const int lo = max(i - 1, 0), cnt = min(i + 1, n - 1) - lo + 1;
+                ok = mbar_wait(pfull + slot, pphase, kPolls);
+                if (i + 1 < n) {
+                    ok = ok && mbar_wait(tempty + fresh, acc_phase, kPolls);
+                    if (++fresh == a.nacc) {
+                        fresh = 0;
+                        acc_phase ^= 1;
                     }
                 }
-                ok = ok && mbar_wait(tempty + acc, acc_phase, kPolls);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
-                const uint32_t td = tmem + acc * a.acc_cols;
-                const bool last = i + 1 == n;
+                const uint32_t x0 = lo32(da) + slot * pstep;
+                const int b = lo - (i - 1), c1 = min(cnt, a.nacc - acc);  // accumulators before the ring wraps
                 if (leader) {
-#pragma unroll
-                    for (int dz = 0; dz < 3; dz++) {
-                        int sl = first + dz;
-                        if (sl >= a.nplanes) sl -= a.nplanes;
-#pragma unroll
-                        for (int r = 0; r < 9; r++) {
-                            const uint32_t x = lo32(da) + sl * pstep + (r % 3) * dxstep + (r / 3) * lstep;
-                            const uint32_t w = lo32(db) + (9 * dz + r) * wstep;
-#pragma unroll
-                            for (int q = 0; q < NP; q++) {
-                                tc_mma(td, x + q * qstep, hi, w + q * wqstep, hi, idesc, (dz + r + q) ? 1u : 0u);
-                                if (CK == 32) tc_mma(td, x + 2, hi, w + 2, hi, idesc, 1);
-                            }
-                        }
-                        // plane z - 1 is done with here; after the last step of a run all three are
-                        if (dz == 0 || last) tc_commit(pempty + sl);
-                    }
-                    tc_commit(tfull + acc);
+                    plane_mmas(x0, acc, b, c1);
+                    if (c1 < cnt) plane_mmas(x0, 0, b + c1, cnt - c1);
+                    tc_commit(pempty + slot);
+                    if (i > 0) tc_commit(tfull + acc);
                 }
                 __syncwarp();
-                first += last ? 3 : 1;
-                if (first >= a.nplanes) first -= a.nplanes;
-                if (++acc == a.nacc) {
-                    acc = 0;
-                    acc_phase ^= 1;
+                if (i > 0 && ++acc == a.nacc) acc = 0;
+                if (++slot == a.nplanes) {
+                    slot = 0;
+                    pphase ^= 1;
                 }
             }
             u += n;
@@ -532,6 +549,18 @@ __global__ void __launch_bounds__(kRingThreads, 1)
         int acc = 0, turn = 0, col = u0 / a.D, z = u0 - col * a.D;
         uint32_t acc_phase = 0;
         bool ok = true;
+        // every accumulator starts from zero (an instruction covers one that begins and two that go on)
+        auto give = [&](int i) {
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(tempty + i)) : "memory");
+        };
+        for (int i = grp; i < a.nacc; i += 2) {
+            for (int c = 0; c < a.bn; c += 16) tc_zero16(trow + i * a.bn + c);
+            give(i);
+        }
         for (int u = u0; u < u1 && ok; u++) {
             if (turn == grp) {
                 ok = __all_sync(0xffffffffu, mbar_wait(tfull + acc, acc_phase, kPolls));
@@ -541,16 +570,12 @@ __global__ void __launch_bounds__(kRingThreads, 1)
                 const size_t vox = ((size_t)z * a.H + y) * a.W + xx;  // used only where valid
                 __nv_bfloat16* out = a.y + vox * a.ldy + n0;
                 const __nv_bfloat16* mask = a.mask + vox * a.ldm + n0;
-                const uint32_t td = trow + acc * a.acc_cols;
+                const uint32_t td = trow + acc * a.bn;
                 for (int c = 0; c < a.bn; c += 16) {
                     float v[16];
                     tc_ld16(td + c, v);
-                    if (c + 16 >= a.bn) {  // the accumulator is in registers
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0)
-                            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(tempty + acc)) : "memory");
-                    }
+                    tc_zero16(td + c);
+                    if (c + 16 >= a.bn) give(acc);  // the accumulator is in registers
                     if (valid) conv_store16(v, a.relu, a.mask ? mask + c : nullptr, out + c);
                 }
             }
@@ -577,8 +602,8 @@ __global__ void __launch_bounds__(kRingThreads, 1)
 }
 
 // ---------------------------------------------------------------------------------------------
-// Weight gradient, general form: dW[t][co][ci] = sum_v dY[v][co] X[v + off_t][ci] = sum_u dY[u - dx][co] X[u + (dz,dy)][ci],
-// all 27 taps in one GEMM: M = (dz, dy) x input channels, N = dx x output channels, K = voxels, split
+// Weight gradient, general form: dW[t][co][ci] = sum_v dY[v][co] X[v + off_t][ci]
+// = sum_u dY[u - dx][co] X[u + (dz,dy)][ci], all 27 taps in one GEMM: M = (dz, dy) x input channels, N = dx x output channels, K = voxels, split
 // over chunks of voxel blocks with a fixed-order sum afterwards.  With the tap's shift shared between
 // the operands a block is fetched as 9 shifted boxes of X and 3 of dY, where 27 shifted boxes of X (and dY
 // once per M tile) took 27 box rows a voxel of the TMA unit's one per cycle (see the file comment).
@@ -736,7 +761,8 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_tc_kernel(const __grid_cons
         const bool leader = elect_one();
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
                                ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-        const uint64_t ad = mnmajor_desc(smem_addr(smem), ra, atom_a), bd = mnmajor_desc(smem_addr(smem) + a_bytes, rb, atom_b);
+        const uint64_t ad = mnmajor_desc(smem_addr(smem), ra, atom_a);
+        const uint64_t bd = mnmajor_desc(smem_addr(smem) + a_bytes, rb, atom_b);
         const uint32_t ahi = hi32(ad), bhi = hi32(bd), stage16 = stage_bytes >> 4, tile16 = tile_bytes >> 4;
         int s = 0, st = 0;
         uint32_t phase = 0, off = 0;
@@ -1095,7 +1121,7 @@ static RingGeom ring_geom(int cin, int cout, int D, int H, int W) {
     // 128 rows past its box: 8 KB of pad follow the weights
     constexpr size_t kRoom = 227 * 1024 - 1024 - 1024 - 8192;
     for (int n = 1; n <= 8 && !a.bn; n++)
-        if (cout % (16 * n) == 0 && cout / n <= 128 && (size_t)27 * (cout / n) * cin * 2 + 3 * plane <= kRoom) {
+        if (cout % (16 * n) == 0 && 3 * (cout / n) <= 256 && (size_t)27 * (cout / n) * cin * 2 + 3 * plane <= kRoom) {
             g.groups = n;
             a.bn = cout / n;
         }
@@ -1105,8 +1131,7 @@ static RingGeom ring_geom(int cin, int cout, int D, int H, int W) {
     a.steps = ytiles * D;
     if ((long long)ytiles * D < 4LL * sms) return g;
     a.steps_per_cta = (a.steps + sms - 1) / sms;
-    a.acc_cols = (a.bn + 31) & ~31;
-    a.nacc = std::min(kMaxAcc, 512 / a.acc_cols);
+    a.nacc = std::min(kMaxAcc, 512 / a.bn);
     a.nplanes = (int)std::min<size_t>(kMaxPlanes, (kRoom - wbytes) / plane);
     g.ctas = (a.steps + a.steps_per_cta - 1) / a.steps_per_cta;
     g.smem = 1024 + a.nplanes * plane + wbytes + 8192;
@@ -1123,7 +1148,7 @@ static cudaError_t launch_ring(RingGeom& g, const void* x, int ldx, const void* 
     const cuuint32_t xb[4] = {(cuuint32_t)g.ck, (cuuint32_t)a.pitch, (cuuint32_t)a.lines, 1};
     const cuuint64_t wd[3] = {(cuuint64_t)a.cin, (cuuint64_t)cout, 27};
     const cuuint64_t ws[2] = {(cuuint64_t)a.cin * 2, (cuuint64_t)a.cin * 2 * cout};
-    const cuuint32_t wb[3] = {(cuuint32_t)g.ck, (cuuint32_t)a.bn, 27};
+    const cuuint32_t wb[3] = {(cuuint32_t)g.ck, (cuuint32_t)a.bn, 1};
     if (kmajor_map(&mx, 4, x, xd, xs, xb) != CUDA_SUCCESS || kmajor_map(&mw, 3, w, wd, ws, wb) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     const int np = a.cin / g.ck;
