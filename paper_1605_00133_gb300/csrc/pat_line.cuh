@@ -591,6 +591,12 @@ __device__ __forceinline__ void line_pass(const LineArgs& a, int tile) {
     if (!PARTS && !late) pdl_wait();
     if (!PARTS && !(a.flags & (LF_TRIGGER_MID | LF_TRIGGER_END))) pdl_trigger();
     constexpr int XN = S::XN;
+    // The two halves (factor, inverse transform, state update, transform) as one loop body: half the code, so fewer
+    // waits for instructions (0.4 cycles of 8 per instruction before).  64x128x128, forward over 400 steps: 7.49 ->
+    // 7.33 ms at L = 128 only, 7.31 at 64 too; 64^3 in one launch a step (pat_step.cuh) 498 -> 451 us over 64 steps.
+    // Shorter lines gain nothing (32^3 293 -> 297 us), L = 256 lost.
+    constexpr bool ROLLED = L == 64 || L == 128;
+    static_assert(!ROLLED || (S::BULK && !S::PFO_ALIAS), "tiles of the rolled form");
     float2 v[B];
     float2 x[XN];
     const bool accum = !PARTS && (a.flags & LF_ACCUM) != 0;
@@ -663,31 +669,65 @@ __device__ __forceinline__ void line_pass(const LineArgs& a, int tile) {
     __syncthreads();  // publishes the mbarrier initialisation (and the parts of the record)
     if (PARTS && record) c.record_sum(c.buf1);
     const bool ok0 = S::STAGE ? c.wait_copy(0) : true;  // the tables
-    c.factor(v, dk[0], kap, a.s_pre);
-    if (!S::BULK) cp_async_wait<1>();  // state 1 has landed; the barrier inside inv() publishes it
-    c.inv(v, x, c.buf0);
-    const bool ok1 = (S::BULK && old1) ? c.wait_copy(1) : true;  // the old state 1
-    c.update(a.st1, c1, !old1 || !ok1, c.pf1, x);
-    if (late) pdl_wait();  // the new spectrum is written by the preceding pass
-    if (a.flags & LF_TRIGGER_MID) pdl_trigger();
     const bool pre = accum && AX != 2;
-    if (S::PFO_ALIAS && pre) {
-        // every thread's state-1 update has read pf1 (written by the bulk copy) before it is reused
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
+    if constexpr (ROLLED) {
+        const float* cs[3] = {c1[0], c1[1], c1[2]};
+        float2* st = a.st1;
+        const float2 *pf = c.pf1, *d = dk[0];
+        float sc = a.s_pre;
+        bool old = old1;
+        int late_copies = ok0 ? 0 : 1;
+#pragma unroll 1
+        for (int h = 0; h < 2; h++) {
+            c.factor(v, d, kap, sc);
+            c.inv(v, x, c.buf0);
+            const bool ok = old ? c.wait_copy(1 + h) : true;
+            if (!ok) late_copies |= 2 << h;
+            c.update(st, cs, !old || !ok, pf, x);
+            if (h == 0) {
+                if (late) pdl_wait();  // the new spectrum is written by the preceding pass
+                if (a.flags & LF_TRIGGER_MID) pdl_trigger();
+                c.prefetch_out(pre);
+            } else {
+                for (int i = 0; i < 3; i++)
+                    if (late_copies & (1 << i)) c.drain(i);
+                cp_async_wait<0>();  // old output; published by the barrier inside fwd()
+            }
+            c.fwd(x, v, c.buf1);
+#pragma unroll
+            for (int i = 0; i < 3; i++) cs[i] = c2[i];
+            st = a.st2;
+            pf = c.pf2;
+            d = dk[1];
+            sc = a.s_mid;
+            old = old2;
+        }
+    } else {
+        c.factor(v, dk[0], kap, a.s_pre);
+        if (!S::BULK) cp_async_wait<1>();  // state 1 has landed; the barrier inside inv() publishes it
+        c.inv(v, x, c.buf0);
+        const bool ok1 = (S::BULK && old1) ? c.wait_copy(1) : true;  // the old state 1
+        c.update(a.st1, c1, !old1 || !ok1, c.pf1, x);
+        if (late) pdl_wait();  // the new spectrum is written by the preceding pass
+        if (a.flags & LF_TRIGGER_MID) pdl_trigger();
+        if (S::PFO_ALIAS && pre) {
+            // every thread's state-1 update has read pf1 (written by the bulk copy) before it is reused
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncthreads();
+        }
+        c.prefetch_out(pre);
+        c.fwd(x, v, c.buf1);
+        c.factor(v, dk[1], kap, a.s_mid);
+        if (!S::BULK) cp_async_wait<1>();  // state 2 likewise (the old output may still be in flight)
+        c.inv(v, x, c.buf0);
+        const bool ok2 = (S::BULK && old2) ? c.wait_copy(2) : true;  // the old state 2
+        c.update(a.st2, c2, !old2 || !ok2, c.pf2, x);
+        if (!ok0) c.drain(0);
+        if (!ok1) c.drain(1);
+        if (!ok2) c.drain(2);
+        cp_async_wait<0>();  // old output; published by the barrier inside fwd()
+        c.fwd(x, v, c.buf1);
     }
-    c.prefetch_out(pre);
-    c.fwd(x, v, c.buf1);
-    c.factor(v, dk[1], kap, a.s_mid);
-    if (!S::BULK) cp_async_wait<1>();  // state 2 likewise (the old output may still be in flight)
-    c.inv(v, x, c.buf0);
-    const bool ok2 = (S::BULK && old2) ? c.wait_copy(2) : true;  // the old state 2
-    c.update(a.st2, c2, !old2 || !ok2, c.pf2, x);
-    if (!ok0) c.drain(0);
-    if (!ok1) c.drain(1);
-    if (!ok2) c.drain(2);
-    cp_async_wait<0>();  // old output; published by the barrier inside fwd()
-    c.fwd(x, v, c.buf1);
     c.factor(v, dk[2], kap, a.s_post);
 
     if (AX == 0 && (a.flags & LF_INJECT) && c.vcol) {

@@ -211,11 +211,11 @@ cudaError_t launch_spread_plane(const Geom& g, const float2* tw_z, const float2*
 }
 
 // Which grids do a step in one launch (pat_step.cuh), by their tiles (CTAs), and in which form.  Loops of 64 steps,
-// three launches a step / one launch of the form for three / for four CTAs an SM:
-//   102 tiles (32^3) 569 / 291 / 291 us, 396 (64^3) 758 / 501 / 545, 534 (16x128x128) 827 / 556 / 610,
-//   788 (128x64x64) 1051 / 980 / 1012, 938 (16x256x128) 1003 / 914 / 913,
-//   1052 (32x128x128) 944 / 966 / 818, 1188 (three volumes of 64^3) 1037 / 1130 / 967,
-//   1584 (four volumes of 64^3) 1109 / - / 1293, 1602 (three of 16x128x128) 1161 / - / 1210.
+// three launches a step / one launch of the form for three / for four CTAs an SM, in us:
+//   102 tiles (32^3) 570 / 293 / 295, 396 (64^3) 731 / 454 / 505, 534 (16x128x128) 766 / 513 / 610,
+//   788 (128x64x64) 1040 / 848 / 960, 938 (16x256x128) 992 / 876 / 872,
+//   1052 (32x128x128) 909 / 929 / 798, 1188 (three volumes of 64^3) 1010 / 1114 / 949,
+//   1584 (four of 64^3) 1086 / 1408 / 1283, 1602 (three of 16x128x128) 1109 / 1251 / 1156.
 // So two rounds of CTAs over the SMs, 2 x 152 x 3 and 2 x 152 x 4: beyond that the passes fill the chip by themselves,
 // and the three spectra read instead of one cost more than the waits.
 int step_residency(const Geom& g) {
