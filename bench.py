@@ -37,7 +37,7 @@ METRIC = "A+A^T pairs/s (64x128x128, 400 steps)"
 
 # (kernel source hash, workload, batch) -> DRAM bytes (read + write) of one forward time step (x, y and
 # z passes), from ncu with the L2 as the run leaves it (--cache-control none)
-STEP_TRAFFIC = {("00f5b3bcbe10", "c2", 1): 4.84e6, ("00f5b3bcbe10", "c4", 1): 672.3e6}
+STEP_TRAFFIC = {("c8ebca04b201", "c2", 1): 4.42e6, ("c8ebca04b201", "c4", 1): 537.0e6}
 UNIT = "pairs/s"
 
 
@@ -499,7 +499,7 @@ def solve_experiment(args, op, f_clean, p0, dev):
 
 def prox_timing(op, x, alpha, iters, reps=5):
     """The TV prox alone at the solver's alpha = eta lam: CUDA events around `reps` calls of `iters`
-    fused primal-dual iterations (one launch each; a call's initial clamp and dual reset included).
+    fused primal-dual iterations (two per launch; a call's initial clamp and dual reset included).
     Algorithmic bytes per voxel and iteration: qbar, the three dual components, q and the input
     read, the dual, q and qbar written, 11 x 4 B = 44 B."""
     import json as _json
@@ -519,12 +519,13 @@ def prox_timing(op, x, alpha, iters, reps=5):
     gbs = 44.0 * voxels / (us * 1e-6) / 1e9
     peaks_path = os.path.join(ROOT, "MEASURED_PEAKS.json")
     peak = float(_json.load(open(peaks_path))["hbm_gbs"]) if os.path.exists(peaks_path) else 6800.0
-    fields = 10 * 4 * voxels  # qbar and the dual (3) in a read and a write buffer each, q, the input
+    fields = 11 * 4 * voxels  # qbar, the dual (3) and q in a read and a write buffer each, the input
     where = ("stay in the 129 MB L2 at this size, so the fraction is of the HBM copy bandwidth, not DRAM "
              "traffic") if fields < 100e6 else "exceed the L2 at this size"
     return {"iters": iters, "us_per_iter": us, "voxels": voxels, "algorithmic_bytes_per_voxel": 44,
             "achieved_gbs": gbs, "frac_of_hbm": gbs / peak,
-            "note": f"one launch per iteration; the prox's fields (10 image-sized FP32 arrays, "
+            "note": f"two iterations per launch, which read and write the fields once (the 44 B are those of "
+                    f"one iteration by itself); the prox's fields (11 image-sized FP32 arrays, "
                     f"{fields / 1e6:.0f} MB) {where}"}
 
 

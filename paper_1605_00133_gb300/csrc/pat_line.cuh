@@ -48,7 +48,7 @@
 //
 // STREAM: the states are loaded and stored evict-first in the L2, for grids whose loop does not fit it.  Their 48
 // bytes per voxel and step then cross DRAM in any case, and left alone they also displace the two spectra and
-// the kappa tables, which are read three times a step.  128x256x256: 672 -> 598 MB of DRAM traffic a step, a
+// the kappa tables, which are read three times a step.  128x256x256: 672 -> 537 MB of DRAM traffic a step, a
 // forward and adjoint over 200 steps 66.7 -> 62.7 ms; 64x128x128 with four volumes a call 7.86 -> 7.33 ms over
 // 100 steps.  Where the loop fits (one volume of 64x128x128) the plain accesses are 0.7 % faster.
 //
