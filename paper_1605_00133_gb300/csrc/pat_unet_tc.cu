@@ -603,7 +603,8 @@ __global__ void __launch_bounds__(kRingThreads, 1)
 
 // ---------------------------------------------------------------------------------------------
 // Weight gradient, general form: dW[t][co][ci] = sum_v dY[v][co] X[v + off_t][ci]
-// = sum_u dY[u - dx][co] X[u + (dz,dy)][ci], all 27 taps in one GEMM: M = (dz, dy) x input channels, N = dx x output channels, K = voxels, split
+// = sum_u dY[u - dx][co] X[u + (dz,dy)][ci], all 27 taps in one GEMM: M = (dz, dy) x input channels, N = dx x
+// output channels, K = voxels, split
 // over chunks of voxel blocks with a fixed-order sum afterwards.  With the tap's shift shared between
 // the operands a block is fetched as 9 shifted boxes of X and 3 of dY, where 27 shifted boxes of X (and dY
 // once per M tile) took 27 box rows a voxel of the TMA unit's one per cycle (see the file comment).
