@@ -318,26 +318,22 @@ __device__ __forceinline__ void head_reduce(double (*red)[18], double* __restric
     if (threadIdx.x < 18) partial[(size_t)blockIdx.x * 18 + threadIdx.x] = red[0][threadIdx.x];
 }
 
-// A running sum as an unevaluated pair of floats: Knuth's two-sum keeps the rounding error of every addition
-// and Dekker's product error (through fma) that of every product, so the sum carries about 47 bits; it
-// becomes a double at the end.  (Adding FP64 products directly, 16 a voxel, is bound by the FP64
-// units, which do about 2 operations per cycle and SM here: 107 us at 1 M voxels, now 35 us.)
-struct FloatPair {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float p, float err) {
-        const float s = hi + p, b = s - hi;
-        lo += ((hi - (s - b)) + (p - b)) + err;
-        hi = s;
-    }
-    __device__ __forceinline__ void add_product(float x, float y) {
-        const float p = x * y;
-        add(p, fmaf(x, y, -p));
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
+// The two BF16 of a word as doubles times 2^-896: their bits moved to a double's places without the change of
+// exponent bias, exact for every finite value (a BF16 subnormal becomes a double's).
+__device__ __forceinline__ double bf16_lo_scaled(uint32_t w) {
+    return __hiloint2double((int)(((w & 0x7fffu) << 13) | ((w << 16) & 0x80000000u)), 0);
+}
+__device__ __forceinline__ double bf16_hi_scaled(uint32_t w) {
+    return __hiloint2double((int)(((w & 0x7fff0000u) >> 3) | (w & 0x80000000u)), 0);
+}
 
-// per block: 16 channel sums of g h, the sum of g, the sum of squared errors.  mask: dh is also taken through
-// the ReLU whose output h is
+// per block: 16 channel sums of g h, the sum of g, the sum of squared errors, in FP64: they cover the range and the
+// precision of a long sum of FP32 products, whatever the data.  mask: dh is also taken through the ReLU whose output h
+// is.  What bounds it: the FP64 units, about 2 operations per cycle and SM here.  16 multiply-adds a voxel are needed,
+// 16 conversions more would be its work too (107 us with them, in the scalar form), so a channel's bits are placed in a
+// double by integer operations, 2^-896 too small, and the factor g carries the 2^896: the products, and so the sums,
+// are those of head_bwd_kernel bit for bit.  A voxel with an infinite or NaN channel is converted.  1 M voxels, with
+// the sum over the blocks: 63 us.  (Sums as pairs of floats take 38, but have FP32's range and 47 bits.)
 __global__ void __launch_bounds__(256) head_bwd8_kernel(const bf16* __restrict__ h, const float* __restrict__ head,
                                                         const float* __restrict__ out, const float* __restrict__ target,
                                                         long long V, bf16* __restrict__ dh, int mask,
@@ -345,32 +341,46 @@ __global__ void __launch_bounds__(256) head_bwd8_kernel(const bf16* __restrict__
     pdl_wait();
     pdl_trigger();
     __shared__ double red[256][18];
-    FloatPair acc[18];
+    double acc[18];
+#pragma unroll
+    for (int k = 0; k < 18; k++) acc[k] = 0.0;
     float w[16];
 #pragma unroll
     for (int c = 0; c < 16; c++) w[c] = __ldca(head + c);
     const double gs = 2.0 / (double)V;
     for (long long v = blockIdx.x * 256LL + threadIdx.x; v < V; v += gridDim.x * 256LL) {
+        const V8 h8[2] = {ld8(h + 16 * v), ld8(h + 16 * v + 8)};
         float f[16];
-        unpack8(ld8(h + 16 * v), f);
-        unpack8(ld8(h + 16 * v + 8), f + 8);
-        const float o = __ldcg(out + v), t = __ldcg(target + v);
-        const float eh = o - t, b = eh - o, el = (o - (eh - b)) - (t + b);  // o - t = eh + el exactly
-        const float g = (float)(gs * ((double)o - (double)t));
-        float d[16];
+        unpack8(h8[0], f);
+        unpack8(h8[1], f + 8);
+        const double e = (double)__ldcg(out + v) - (double)__ldcg(target + v);
+        const float g = (float)(gs * e);
+        const double gd = (double)g;
+        float d[16], odd = 0.f;
 #pragma unroll
         for (int c = 0; c < 16; c++) {
-            acc[c].add_product(g, f[c]);
+            odd = fmaf(f[c], 0.f, odd);  // NaN if any channel is not finite
             d[c] = (!mask || f[c] > 0.f) ? g * w[c] : 0.f;
         }
         st8(dh + 16 * v, pack8(d));
         st8(dh + 16 * v + 8, pack8(d + 8));
-        acc[16].add(g, 0.f);
-        const float p = eh * eh;
-        acc[17].add(p, fmaf(2.f * eh, el, fmaf(eh, eh, -p)));
+        if (odd == 0.f) {
+            const double gb = gd * 0x1p896;  // finite where g is
+            const uint32_t* u = reinterpret_cast<const uint32_t*>(h8);
+#pragma unroll
+            for (int c = 0; c < 16; c += 2) {
+                acc[c] = fma(gb, bf16_lo_scaled(u[c / 2]), acc[c]);
+                acc[c + 1] = fma(gb, bf16_hi_scaled(u[c / 2]), acc[c + 1]);
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < 16; c++) acc[c] = fma(gd, (double)f[c], acc[c]);
+        }
+        acc[16] += gd;
+        acc[17] = fma(e, e, acc[17]);
     }
 #pragma unroll
-    for (int k = 0; k < 18; k++) red[threadIdx.x][k] = acc[k].value();
+    for (int k = 0; k < 18; k++) red[threadIdx.x][k] = acc[k];
     head_reduce(red, partial);
 }
 __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16* __restrict__ h, const float* __restrict__ head,
@@ -387,11 +397,11 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16* __restrict__ 
 #pragma unroll
         for (int c = 0; c < 16; c++) {
             const float hv = __bfloat162float(h[v * 16 + c]);
-            acc[c] += (double)g * hv;
+            acc[c] = fma((double)g, (double)hv, acc[c]);
             dh[v * 16 + c] = __float2bfloat16((!mask || hv > 0.f) ? g * head[c] : 0.f);
         }
-        acc[16] += g;
-        acc[17] += e * e;
+        acc[16] += (double)g;
+        acc[17] = fma(e, e, acc[17]);
     }
     for (int k = 0; k < 18; k++) red[threadIdx.x][k] = acc[k];
     head_reduce(red, partial);
