@@ -161,6 +161,27 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, float* v) {
     for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
 }
 
+// the same of two groups of columns, in flight together
+__device__ __forceinline__ void tc_ld16x2(uint32_t ta, uint32_t tb, float* v, float* u) {
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, "
+        "[%32];\n\t"
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, "
+        "%31}, [%33];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(ta), "r"(tb));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+        v[i] = __uint_as_float(r[i]);
+        u[i] = __uint_as_float(r[16 + i]);
+    }
+}
+
 // zeros into 16 consecutive FP32 columns of this thread's tensor-memory lane (tc_wait_st() before they are relied on)
 __device__ __forceinline__ void tc_zero16(uint32_t taddr) {
     asm volatile(
@@ -617,6 +638,8 @@ __global__ void __launch_bounds__(kRingThreads, 1)
 // memory with their N columns and three stages of shared memory), so one fetch of a block serves them all.
 // The boxes of a stage are issued by the lanes of the producer warp together, each its own (coordinates and
 // destinations are fixed per lane but for the block).
+// Accuracy: one accumulator sums a CTA's share of the voxels, truncating, so the error grows with the volume: 64 -> 64
+// and 192 -> 64 channels at 16x32x32 voxels 1.9e-7 and 5.0e-7 with ReLU'd operands, 64 -> 64 at 64x128x128 3.4e-5.
 // ---------------------------------------------------------------------------------------------
 
 constexpr int kKB = 64;  // voxels per K block
@@ -835,9 +858,18 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_tc_kernel(const __grid_cons
 // rows a voxel instead of 9 blocks + 3.  An M group that needs two of the three dy fetches R + 1 lines.
 // Rows of the last M tile beyond the 9 blocks atoms multiply whatever follows in shared memory and are not used.
 // What bounds it: the MMAs with few channels (two M tiles of N = 48 for 16 -> 16: 49 cycles each), the TMA unit with
-// more.  With the partial products written 512 bytes a warp (16 bytes a lane, 192 or more apart, before) the
-// whole gradient took, before -> now: 64x128x128 voxels 16 -> 16 channels 69.9 -> 35.0 us, 48 -> 16
-// 145 -> 92; 32x64x64 voxels 32 -> 32 31.5 -> 20.7, 96 -> 32 49.5 -> 31.0.
+// more.  The whole gradient took with wgrad_tc_kernel (its partial products written 16 bytes a lane, 192 or more apart) ->
+// now: 64x128x128 voxels 16 -> 16 channels 69.9 -> 32 us, 48 -> 16 145 -> 64; 32x64x64 voxels 32 -> 32 31.5 -> 16,
+// 96 -> 32 49.5 -> 28.
+// Accuracy: the tensor core truncates as it adds, so a sum of n voxels of one sign comes out low by about 1.3e-9 n of
+// its value (7168 voxels 9.1e-6, 14144 2.0e-5).  So K blocks go to two accumulators in turn where tensor memory holds
+// two, and after kChain voxels in each, or at the end, the epilogue adds them up, rounding to nearest, and to what
+// earlier segments left in the partial product.  ReLU'd operands, relative error against FP64 of one accumulator to the
+// end -> now: 64x128x128 voxels 16 -> 16 channels 9.1e-6 -> 3.8e-6 (1 us more), 48 -> 16 8.9e-6 -> 3.8e-6 (with its
+// tiles in two groups and chains twice as long 2.0e-5); 32x64x64 voxels 16 -> 32 9.5e-7 -> 4.1e-7; 128x256x256 voxels
+// 16 -> 16 1.0e-4 -> 8.8e-6 (200 -> 218 us).
+constexpr int kChain = 7168;  // most voxels summed by one accumulator: 448 MMAs
+
 struct WlineArgs {
     float4* partial;    // as above; rows in the order (dy, dz, channel), columns (1 - dx, output channel)
     int cb, wa, bn;     // channel blocks, their channels; output channels
@@ -845,6 +877,7 @@ struct WlineArgs {
     int bx, R, lines;   // voxels per line, lines of a block, lines of X fetched for it
     int tx, ty, nkb;    // blocks along x and y, in all
     int kb_per_cta;
+    int nset, seg;      // accumulators taking K blocks in turn; K blocks after which they are added up
     int nstage;
     uint32_t stage_bytes, x_bytes, bar_off;
     uint32_t tmem_cols;
@@ -859,6 +892,52 @@ __device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, i
         : "memory");
 }
 
+// wgrad_store of the sum of nset <= 2 accumulators set_cols columns apart, N a multiple of 48.  more: added to what is
+// there (this thread's own, of the segment before), 12 loads in flight.
+__device__ __forceinline__ void wgrad_store_sum(uint32_t taddr, int nset, int set_cols, int N, bool more, float4* out) {
+    for (int c0 = 0; c0 < N; c0 += 48) {
+        float4* p = out + (size_t)(c0 / 4) * kBM;
+        float4 o[12];
+        if (more) {
+#pragma unroll
+            for (int i = 0; i < 12; i++) o[i] = p[i * kBM];
+        }
+#pragma unroll
+        for (int h = 0; h < 3; h++) {
+            float v[16];
+            if (nset > 1) {
+                float u[16];
+                tc_ld16x2(taddr + (uint32_t)(c0 + 16 * h), taddr + (uint32_t)(set_cols + c0 + 16 * h), v, u);
+#pragma unroll
+                for (int i = 0; i < 16; i++) v[i] += u[i];
+            } else {
+                tc_ld16(taddr + (uint32_t)(c0 + 16 * h), v);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                float4 t = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                if (more) {
+                    const float4 w = o[4 * h + i];
+                    t = make_float4(w.x + t.x, w.y + t.y, w.z + t.z, w.w + t.w);
+                }
+                p[(4 * h + i) * kBM] = t;
+            }
+        }
+    }
+}
+
+// Where the MMA issuer is: the segment, its K block, and the accumulator of that.
+struct WgradTurn {
+    int i = 0, set = 0, segment = 0;
+    __device__ __forceinline__ void next(int nset, int seg) {
+        if (++set == nset) set = 0;
+        if (++i == seg) {
+            i = set = 0;
+            segment++;
+        }
+    }
+};
+
 template <int KS>  // bx / 16
 __global__ void __launch_bounds__(kThreads, 1) wgrad_line_kernel(const __grid_constant__ CUtensorMap tmx,
                                                                  const __grid_constant__ CUtensorMap tmd,
@@ -867,12 +946,13 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_line_kernel(const __grid_co
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t ra = 2u * a.wa, rb = 2u * a.bn;  // row bytes = swizzle widths
     const uint32_t unit = a.bx * ra;                // one atom
-    const int N = 3 * a.bn, ncols = (N + 31) & ~31, nstage = a.nstage;
+    const int N = 3 * a.bn, ncols = (N + 31) & ~31, set_cols = a.mt * ncols, nstage = a.nstage;
     const uint32_t d_bytes = a.R * (a.bx + 2) * rb;
     unsigned long long* full = reinterpret_cast<unsigned long long*>(smem + a.bar_off);
     unsigned long long* empty = full + nstage;
     unsigned long long* done = empty + nstage;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    unsigned long long* drained = done + 1;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drained + 1);
     int* counts = reinterpret_cast<int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -892,6 +972,7 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_line_kernel(const __grid_co
             mbar_init(empty + s, 1);
         }
         mbar_init(done, 1);
+        mbar_init(drained, 4);  // one arrival per epilogue warp
         mbar_fence_init();
         counts[0] = counts[1] = counts[2] = 0;
     }
@@ -942,16 +1023,19 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_line_kernel(const __grid_co
         const uint32_t tile16 = (kBM / a.wa) * unit >> 4, aline16 = 3 * a.cb * unit >> 4, bline16 = (a.bx + 2) * rb >> 4;
         int s = 0, st = 0;
         uint32_t phase = 0, off = 0;
+        WgradTurn w;
         for (; s < nkb; s++) {
-            if (!__all_sync(0xffffffffu, mbar_wait(full + st, phase, kPolls))) {
+            bool ok = mbar_wait(full + st, phase, kPolls);
+            if (w.i == 0 && s > 0) ok = ok && mbar_wait(drained, (w.segment - 1) & 1, kPolls);
+            if (!__all_sync(0xffffffffu, ok)) {
                 if (leader) counts[2] = 1;
                 break;
             }
             tc_fence_after();
-            uint32_t al = lo32(ad) + off, td = tmem;
+            uint32_t al = lo32(ad) + off, td = tmem + w.set * set_cols;
             const uint32_t bl = lo32(bd) + off;
             for (int t = 0; t < mt; t++, al += tile16, td += ncols) {
-                uint32_t alo = al, blo = bl, on = s > 0 ? 1u : 0u;
+                uint32_t alo = al, blo = bl, on = w.i >= a.nset ? 1u : 0u;
                 for (int r = 0; r < a.R; r++, alo += aline16, blo += bline16) {
                     // 16 voxel rows: the starts move by 16 rows of each operand
 #pragma unroll
@@ -960,8 +1044,12 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_line_kernel(const __grid_co
                     on = 1u;
                 }
             }
-            if (leader) tc_commit(empty + st);
+            if (leader) {
+                tc_commit(empty + st);
+                if (w.i + 1 == a.seg && s + 1 < nkb) tc_commit(done);
+            }
             __syncwarp();
+            w.next(a.nset, a.seg);
             off += stage16;
             if (++st == nstage) {
                 st = 0;
@@ -973,15 +1061,30 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_line_kernel(const __grid_co
             counts[1] = s;
             tc_commit(done);
         }
-    } else if (warp >= 2) {
-        const bool ok = mbar_wait(done, 0, kPolls);
-        if (!ok) counts[2] = 1;
         __syncwarp();
-        tc_fence_after();
+        // every MMA has finished before the tensor memory is freed (a loop that ended at nkb is in its last segment)
+        mbar_wait(done, (s == nkb ? (nkb - 1) / a.seg : w.segment) & 1, kPolls);
+    } else if (warp >= 2) {
+        // epilogue: adds up the accumulators of each segment once it is done, and hands them back
         const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
-        for (int t = 0; t < mt; t++)
-            wgrad_store(trow + (uint32_t)(t * ncols), N,
-                        a.partial + ((size_t)chunk * a.mtiles + mtile0 + t) * (N / 4) * kBM + 32 * (warp & 3) + lane);
+        float4* out = a.partial + ((size_t)chunk * a.mtiles + mtile0) * (N / 4) * kBM + 32 * (warp & 3) + lane;
+        for (int j = 0; j * a.seg < nkb; j++) {
+            bool ok = mbar_wait(done, j & 1, kPolls);
+            if (!ok) counts[2] = 1;
+            ok = ok && !*const_cast<volatile int*>(counts + 2);  // set before `done` if the issuer gave up
+            if (!__all_sync(0xffffffffu, ok)) break;
+            tc_fence_after();
+            const int ns = min(a.nset, min(a.seg, nkb - j * a.seg));
+            for (int t = 0; t < mt; t++)
+                if (ns > 1 || j > 0)
+                    wgrad_store_sum(trow + t * ncols, ns, set_cols, N, j > 0, out + (size_t)t * (N / 4) * kBM);
+                else
+                    wgrad_store(trow + t * ncols, N, out + (size_t)t * (N / 4) * kBM);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(drained)) : "memory");
+        }
     }
     tc_fence_before();
     __syncthreads();
@@ -989,7 +1092,6 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_line_kernel(const __grid_co
         if (threadIdx.x == 0) {
             atomicOr(&g_unet_err, 1);
             for (int s = counts[1]; s < counts[0]; s++) mbar_wait(full + s % nstage, (s / nstage) & 1, kPolls);
-            mbar_wait(done, 0, kPolls);
         }
         __syncthreads();
     }
@@ -1287,7 +1389,7 @@ static WgradGeom wgrad_geom(int cin, int cout, int D, int H, int W) {
 // atom of dY (16 or 32), whose N columns would have no single leading byte offset, or over 96 input channels, of which
 // three stages hold too few lines.
 struct WlineGeom {
-    int wa, cb, mtiles, mt, mgroups, span, bx, R, tx, ty, nkb, nstage, kb_per_cta, nchunk;
+    int wa, cb, mtiles, mt, mgroups, span, bx, R, tx, ty, nkb, nset, seg, nstage, kb_per_cta, nchunk;
     uint32_t tmem_cols, x_bytes, stage_bytes, bar_off;
     size_t smem;
 };
@@ -1299,19 +1401,20 @@ static WlineGeom wline_geom(int cin, int cout, int D, int H, int W) {
     g.cb = cin / g.wa;
     const int per_tile = kBM / g.wa, N = 3 * cout, ncols = (N + 31) & ~31;
     g.mtiles = (9 * cin + kBM - 1) / kBM;
-    // Up to three M tiles a CTA.  With all four of 48 channels in one (and twice the chunks) the sums come out
-    // closer to 64 bits, but 1.7e-5 from those of half the chunks: the tensor core truncates as it adds.
-    g.mgroups = (g.mtiles + 2) / 3;
+    // Up to four M tiles a CTA, so that 48 channels are one group, whose lines are fetched once: 48 -> 16 channels at
+    // 64x128x128 64 us, in two groups of two tiles 87 (and the same accuracy).
+    g.mgroups = (g.mtiles + 3) / 4;
     g.mt = (g.mtiles + g.mgroups - 1) / g.mgroups;
     for (int i = 0; i < g.mgroups; i++) {
         const int a0 = i * g.mt * per_tile, a1 = std::min((i + 1) * g.mt * per_tile, 9 * g.cb) - 1;
         g.span = std::max(g.span, a1 / (3 * g.cb) - a0 / (3 * g.cb));
     }
+    g.nset = std::min(2, 512 / (g.mt * ncols));  // one CTA an SM: all of its tensor memory
     g.tmem_cols = 64;
-    while ((int)g.tmem_cols < g.mt * ncols) g.tmem_cols *= 2;
+    while ((int)g.tmem_cols < g.nset * g.mt * ncols) g.tmem_cols *= 2;
     // The block shape with the least time of TMA unit (a box row a cycle) or MMAs, over the volume padded to whole
-    // blocks; 200 cycles for what a stage costs besides.  48 -> 16 channels at 64x128x128: 16 voxels x 13 lines
-    // 92 us, 32 x 4 100, 64 x 2 117.
+    // blocks; 200 cycles for what a stage costs besides.  48 -> 16 channels at 64x128x128, in two groups of tiles:
+    // 16 voxels x 13 lines 92 us, 32 x 4 100, 64 x 2 117.
     constexpr int kSmem = 227 * 1024 - 1024 - 256;
     double best = 0;
     for (int bx = 16; bx <= 64 && bx < W + 16; bx += 16)
@@ -1346,8 +1449,9 @@ static WlineGeom wline_geom(int cin, int cout, int D, int H, int W) {
     const long long nkb = (long long)g.tx * g.ty * D;
     if (nkb > INT_MAX) return g;
     g.nkb = (int)nkb;
+    g.seg = g.nset * (kChain / (g.bx * g.R));
     // one CTA an SM: more than half of its shared memory
-    g.smem = std::max<size_t>(1024 + g.bar_off + (2 * g.nstage + 1) * 8 + 4 + 16, 233472 / 2);
+    g.smem = std::max<size_t>(1024 + g.bar_off + (2 * g.nstage + 2) * 8 + 4 + 16, 233472 / 2);
     const int want = std::max(1, 152 / g.mgroups), least = std::max(1, 256 / (g.bx * g.R));
     g.kb_per_cta = std::max((g.nkb + want - 1) / want, least);
     g.nchunk = (g.nkb + g.kb_per_cta - 1) / g.kb_per_cta;
@@ -1406,6 +1510,8 @@ static cudaError_t wgrad_line(EncodeTiled enc, const WlineGeom& g, const void* x
     a.ty = g.ty;
     a.nkb = g.nkb;
     a.kb_per_cta = g.kb_per_cta;
+    a.nset = g.nset;
+    a.seg = g.seg;
     a.nstage = g.nstage;
     a.stage_bytes = g.stage_bytes;
     a.x_bytes = g.x_bytes;
