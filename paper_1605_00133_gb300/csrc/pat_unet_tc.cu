@@ -1143,6 +1143,15 @@ __global__ void __launch_bounds__(32 * S) wgrad_sum_kernel(const float4* __restr
     dw[((size_t)(3 * tap_row + d) * cout + g * bn + r - j * bn) * cin + ci] = t;
 }
 
+// A kernel's cap on dynamic shared memory is one for all host threads: always set to the most any shape takes (all of an
+// SM's but for what the kernel declares itself), so that no thread lowers it between another's call and its launch.
+constexpr size_t kSmemCap = 227 * 1024, kRingSmemCap = 226 * 1024;
+template <typename... P>
+cudaError_t raise_smem(void (*kernel)(P...), size_t cap, size_t smem) {
+    if (smem > cap) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cap);
+}
+
 template <typename... P, typename... A>
 cudaError_t launch(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
     const cudaError_t e = launch_pdl(kernel, grid, threads, smem, st, args...);
@@ -1178,7 +1187,7 @@ cudaError_t launch_ck(const CUtensorMap& mx, const CUtensorMap& mw, const ConvTc
     const size_t max_ctas = 512 / a.tmem_cols;
     const size_t floor_smem = 233472 / (max_ctas + 1) + 1;
     if (smem < floor_smem) smem = floor_smem;
-    cudaError_t e = cudaFuncSetAttribute(conv3_tc_kernel<CK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_smem(conv3_tc_kernel<CK>, kSmemCap, smem);
     if (e != cudaSuccess) return e;
     return launch(conv3_tc_kernel<CK>, dim3(tiles, (unsigned)(a.cout / a.bn)), kThreads, smem, st, mx, mw, a);
 }
@@ -1260,7 +1269,7 @@ static cudaError_t launch_ring(RingGeom& g, const void* x, int ldx, const void* 
                         : np == 2  ? conv3_ring_kernel<16, 2>
                         : np == 3  ? conv3_ring_kernel<16, 3>
                                    : conv3_ring_kernel<16, 4>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+    cudaError_t e = raise_smem(kernel, kRingSmemCap, g.smem);
     if (e != cudaSuccess) return e;
     return launch(kernel, dim3((unsigned)g.ctas, (unsigned)g.groups), kRingThreads, g.smem, st, mx, mw, a);
 }
@@ -1519,7 +1528,7 @@ static cudaError_t wgrad_line(EncodeTiled enc, const WlineGeom& g, const void* x
     a.tmem_cols = g.tmem_cols;
     const auto kernel = g.bx == 64 ? wgrad_line_kernel<4> : g.bx == 48 ? wgrad_line_kernel<3>
                         : g.bx == 32 ? wgrad_line_kernel<2> : wgrad_line_kernel<1>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+    cudaError_t e = raise_smem(kernel, kSmemCap, g.smem);
     if (e != cudaSuccess) return e;
     e = launch(kernel, dim3((unsigned)g.mgroups, (unsigned)g.nchunk), kThreads, g.smem, st, mx, md, a);
     if (e != cudaSuccess) return e;
@@ -1581,7 +1590,7 @@ cudaError_t wgrad_tc(const void* x, int ldx, int cin, const void* dy, int ldy, i
     a.kb_per_cta = g.kb_per_cta;
     a.nstage = g.nstage;
     a.tmem_cols = g.tmem_cols;
-    cudaError_t e = cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+    cudaError_t e = raise_smem(wgrad_tc_kernel, kSmemCap, g.smem);
     if (e != cudaSuccess) return e;
     e = launch(wgrad_tc_kernel, dim3((unsigned)(g.mgroups * g.ngroups), (unsigned)g.nchunk), kThreads, g.smem, st, mx,
                    md, a);
