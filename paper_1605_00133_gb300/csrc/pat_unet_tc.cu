@@ -1174,6 +1174,10 @@ EncodeTiled encoder() {
             q == cudaDriverEntryPointSuccess)
             fn = reinterpret_cast<EncodeTiled>(p);
     });
+    // a map is encoded in the thread's current context, which a thread that has none yet gets here (also under capture)
+    thread_local bool bound = false;
+    int device;
+    if (!bound) bound = cudaGetDevice(&device) == cudaSuccess && cudaSetDevice(device) == cudaSuccess;
     return fn;
 }
 

@@ -71,3 +71,39 @@ def test_threads_with_different_shapes():
             if grad:
                 assert torch.equal(results[i][1], want[i][1])
         _lib.check(L.pat_unet_device_status(st))
+
+
+def test_a_thread_whose_first_call_is_a_layer():
+    """Nothing else of CUDA has run in the thread: the call finds the device's context by itself."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1605_00133_gb300 import _lib
+    L, dev = _lib.load(), torch.device("cuda", 0)
+    x, w = torch.ones((64, 16), device=dev).bfloat16(), torch.ones((27, 16, 16), device=dev).bfloat16()
+    y, dw = torch.zeros((64, 16), device=dev).bfloat16(), torch.zeros((27, 16, 16), device=dev)
+    scratch, z = torch.empty(L.pat_unet_wgrad_scratch(16, 16, 4, 4, 4), device=dev), torch.zeros_like(y)
+    torch.cuda.synchronize()
+    status = []
+
+    def conv():
+        status.append(L.pat_unet_conv3(x.data_ptr(), 16, 16, w.data_ptr(), 16, y.data_ptr(), 16, 4, 4, 4, 0, None))
+
+    def grad():
+        status.append(L.pat_unet_conv3_wgrad(x.data_ptr(), 16, 16, x.data_ptr(), 16, 16, 4, 4, 4, scratch.data_ptr(),
+                                             dw.data_ptr(), None))
+    def captured():
+        stream, graph = torch.cuda.Stream(dev), torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            status.append(L.pat_unet_conv3(x.data_ptr(), 16, 16, w.data_ptr(), 16, z.data_ptr(), 16, 4, 4, 4, 0,
+                                           stream.cuda_stream))
+        graph.replay()
+        torch.cuda.synchronize()
+    for f in (conv, grad, captured):
+        t = threading.Thread(target=f)
+        t.start()
+        t.join()
+    torch.cuda.synchronize()
+    assert status == [0, 0, 0] and torch.equal(y, z)
+    assert float(y[21, 0]) == 27 * 16 and float(dw[13, 0, 0]) == 64  # an inner voxel; the centre tap
