@@ -239,8 +239,8 @@ __global__ void __launch_bounds__(32 * kTvWarps) tv_step_kernel(TvStep a) {
 // and 18 rows for 16), and three planes more than a run stores.  Neighbours along x and y come through
 // shared memory (two barriers per plane for both iterations), along z through registers; a plane's inputs
 // are fetched while the one before is computed.  Per voxel the operations are tv_step_kernel's, in the same
-// order, so the results are the same bit for bit.  20 iterations of 128x256x256 2193 -> 1113 us,
-// 50 of 64x128x128 829 -> 425 us.
+// order, so the results are the same bit for bit.  20 iterations of 128x256x256 2193 -> 1101 us,
+// 50 of 64x128x128 829 -> 411 us.
 struct TvStep2 {
     const float* qb_in;
     float* qb_out;
@@ -274,7 +274,10 @@ struct TvIn4 {
 // "Computation of elementary functions on the IBM RISC System/6000", 1990).  Compared with sqrtf and the division
 // on the device: equal for all 2^24 mantissas and for 2^32 random quotients (12 differ without the step on
 // 1 / g, for 2 % of the time).  The bounds on the radius keep the residuals' exponents in range for every norm
-// that is scaled.  The norm comes out as NaN where its square is 0, infinite or NaN, of which the infinite one
+// that is scaled.  A numerator v below 2^-102 has a residual below the subnormals' spacing: such quotients (the front of
+// an image that spreads into zeros decays through them) are divided after all, four at a time in a branch that is
+// rarely taken (50 iterations of 64x128x128 with it 411 us, without 425: the division's loop is also cut in two).
+// The norm comes out as NaN where its square is 0, infinite or NaN, of which the infinite one
 // scales by 0 and the others by 1, as in tv_scale.
 constexpr float kTvRadiusMin = 1e-15f, kTvRadiusMax = 1e15f;  // outside, or NaN: one iteration at a time
 __device__ __forceinline__ float tv_scale_fast(float n, float alpha) {
@@ -294,6 +297,9 @@ __device__ __forceinline__ float tv_divide(float v, float d, float inv) {
     const float q = v * inv, rem = fmaf(-q, d, v);
     return rem == rem ? fmaf(rem, inv, q) : q;  // infinite v
 }
+
+constexpr unsigned kTvTiny = 2u * 0x0d800000u;  // twice the bits of 2^-100
+__device__ __noinline__ float4 tv_divide4(float4 v, float d) { return make_float4(v.x / d, v.y / d, v.z / d, v.w / d); }
 
 __device__ __forceinline__ float& at4(float4& v, int i) { return reinterpret_cast<float*>(&v)[i]; }
 __device__ __forceinline__ float at4(const float4& v, int i) { return reinterpret_cast<const float*>(&v)[i]; }
@@ -368,6 +374,8 @@ __global__ void __launch_bounds__(kTv2Threads, 1) tv_step2_kernel(TvStep2 a) {
                       const float4& dyl, const float4& dx, float dxl, float4& qn, float4& qb) {
         const float tau = a.tau[k], theta = a.theta[k];
         const bool zn = z + 1 < a.nz;
+        float4 num, quo;
+        unsigned least = ~0u;  // twice the least magnitude but 0, less 1
 #pragma unroll
         for (int i = 0; i < 4; i++) {
             float gt = 0.f;
@@ -377,7 +385,14 @@ __global__ void __launch_bounds__(kTv2Threads, 1) tv_step2_kernel(TvStep2 a) {
             if (y > 0) gt += at4(dyl, i);
             if (i < 3 || !xlast) gt -= at4(dx, i);
             if (i > 0 || x > 0) gt += i > 0 ? at4(dx, i - 1) : dxl;
-            float v = tv_divide(fmaf(-tau, gt, fmaf(tau, at4(p, i), at4(q, i))), 1.f + tau, a.inv[k]);
+            at4(num, i) = fmaf(-tau, gt, fmaf(tau, at4(p, i), at4(q, i)));
+            at4(quo, i) = tv_divide(at4(num, i), 1.f + tau, a.inv[k]);
+            least = min(least, 2u * __float_as_uint(at4(num, i)) - 1u);
+        }
+        if (least < kTvTiny) quo = tv_divide4(num, 1.f + tau);
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            float v = at4(quo, i);
             if (a.nonneg) v = fmaxf(0.f, v);
             at4(qn, i) = v;
             at4(qb, i) = fmaf(theta, v - at4(q, i), v);
