@@ -43,14 +43,15 @@ pat_status pat_unet_conv3_masked(const void* x, int32_t ldx, int32_t cin, const 
                                  void* cuda_stream);
 
 /* Synchronises cuda_stream, then reads and clears the device word in which the tensor-core
- * convolutions record a bounded wait that gave up: PAT_OK, or PAT_ERR_TIMEOUT (the outputs of the
- * convolutions since the last check are invalid). */
+ * convolutions and weight gradients record a bounded wait that gave up: PAT_OK, or PAT_ERR_TIMEOUT
+ * (their outputs since the last check are invalid). */
 pat_status pat_unet_device_status(void* cuda_stream);
 
 /* Test hook for that failure path (no counterpart in the paper), process-wide: while
- * stop_after_stage >= 0, the convolutions (pat_unet_conv3) issue the TMA copies of only their first
- * stop_after_stage K steps and give up waiting for the next after `polls` polls (0: the default);
- * nothing is left in flight, each CTA frees its tensor memory and exits, the outputs are invalid and
+ * stop_after_stage >= 0, the convolutions and weight gradients issue the TMA copies of only their
+ * first stop_after_stage K steps (the convolution ring of few channels and large volumes: input
+ * planes) per CTA and give up waiting for the next after `polls` polls (0: the default); nothing is
+ * left in flight, each CTA frees its tensor memory and exits, the outputs are invalid and
  * pat_unet_device_status reports PAT_ERR_TIMEOUT.  stop_after_stage = -1 restores normal operation. */
 pat_status pat_unet_debug_copy_fault(int32_t stop_after_stage, int32_t polls);
 

@@ -39,6 +39,7 @@
 #include <algorithm>
 #include <climits>
 #include <mutex>
+#include <type_traits>
 
 #include "pat_fft.cuh"
 
@@ -53,9 +54,23 @@ constexpr int kBM = 128;
 constexpr int kThreads = 192;
 constexpr int kPolls = 1 << 20;  // bounded waits: each poll suspends for at most about a microsecond
 
-// test hook of the convolution's failure path (pat_unet_debug_copy_fault): process-wide
+// test hook of the kernels' failure paths (pat_unet_debug_copy_fault): process-wide
 int g_stop_after = -1;
 int g_polls = kPolls;
+struct CopyFault {
+    int stop_after;  // the producer issues only stages (of conv3_ring_kernel: input planes) < stop_after (< 0: all)
+    int polls;       // poll limit of the waits for what the hook leaves out
+    // ON: whether the kernel reads the hook.  The ring and the gradient by lines have a form that does not: limits that
+    // vary cost them up to 5 % (16 -> 16 channels at 64x128x128 30.7 -> 32.1 us).
+    template <bool ON = true>
+    __device__ __forceinline__ bool out(int s) const {
+        return ON && stop_after >= 0 && s >= stop_after;
+    }
+    template <bool ON = true>
+    __device__ __forceinline__ int limit(int s) const {
+        return out<ON>(s) ? polls : kPolls;
+    }
+};
 
 struct ConvTcArgs {
     __nv_bfloat16* y;
@@ -67,8 +82,7 @@ struct ConvTcArgs {
     int tx, ty;         // tiles along x and y
     int relu;
     uint32_t tmem_cols;
-    int stop_after;     // test hook: the producer issues only stages < stop_after (< 0: all)
-    int polls;          // poll limit of the wait for the first stage the test hook leaves out
+    CopyFault fault;
 };
 
 // shared-memory matrix descriptor of a K-major operand tile: rows of `row_bytes` (= the swizzle
@@ -279,7 +293,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(const __grid_cons
         int s = 0, st = 0, c0 = 0, t = 0, dx = -1, dy = -1, dz = -1;
         uint32_t phase = 1;  // a fresh empty barrier's preceding phase counts as complete
         for (; s < S; s++) {
-            if (a.stop_after >= 0 && s >= a.stop_after) break;  // test hook: nothing more is issued
+            if (a.fault.out(s)) break;  // test hook: nothing more is issued
             if (!mbar_wait(empty + st, phase, kPolls)) {
                 counts[2] = 1;
                 break;
@@ -314,9 +328,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv3_tc_kernel(const __grid_cons
         int s = 0, st = 0, c0 = 0;
         uint32_t phase = 0, lo = lo0;
         for (; s < S; s++) {
-            // the test hook's short limit applies only to the first stage it leaves out
-            const int lim = (a.stop_after >= 0 && s >= a.stop_after) ? a.polls : kPolls;
-            if (!__all_sync(0xffffffffu, mbar_wait(full + st, phase, lim))) {
+            if (!__all_sync(0xffffffffu, mbar_wait(full + st, phase, a.fault.limit(s)))) {
                 if (leader) counts[2] = 1;
                 break;
             }
@@ -420,9 +432,10 @@ struct ConvRingArgs {
     int nplanes, nacc;        // ring of input planes, of accumulators (bn columns each)
     uint32_t box_bytes;       // one part of one copy of a plane
     uint32_t dxstep;          // from tap dx to dx + 1, in 16-byte units: a copy or a row
+    CopyFault fault;
 };
 
-template <int CK, int NP>  // NP parts of CK input channels
+template <int CK, int NP, bool FAULT>  // NP parts of CK input channels; FAULT: with the test hook
 __global__ void __launch_bounds__(kRingThreads, 1)
     conv3_ring_kernel(const __grid_constant__ CUtensorMap tmx, const __grid_constant__ CUtensorMap tmw, ConvRingArgs a) {
     extern __shared__ uint8_t smem_raw[];
@@ -476,9 +489,9 @@ __global__ void __launch_bounds__(kRingThreads, 1)
         int p = 0, slot = 0;
         uint32_t phase = 1;  // a fresh empty barrier's preceding phase counts as complete
         bool ok = true;
-        for (int u = u0; u < u1 && ok;) {
+        for (int u = u0; u < u1 && ok && !a.fault.out<FAULT>(p);) {
             const int col = u / a.D, z0 = u - col * a.D, n = min(u1 - u, a.D - z0);
-            for (int z = z0 - 1; z <= z0 + n; z++, p++) {
+            for (int z = z0 - 1; z <= z0 + n && !a.fault.out<FAULT>(p); z++, p++) {
                 if (!mbar_wait(pempty + slot, phase, kPolls)) {
                     ok = false;
                     break;
@@ -522,14 +535,15 @@ __global__ void __launch_bounds__(kRingThreads, 1)
         };
         bool ok = mbar_wait(&wfull, 0, kPolls);
         int slot = 0, acc = 0;  // ring slots of the plane and of its first output
+        int p = 0;              // planes so far
         uint32_t pphase = 0, acc_phase = 0;
         int fresh = 0;          // accumulator of the next output to begin
         for (int u = u0; u < u1 && ok;) {
             const int col = u / a.D, z0 = u - col * a.D, n = min(u1 - u, a.D - z0);
-            for (int i = -1; i <= n; i++) {
+            for (int i = -1; i <= n; i++, p++) {
                 // plane z0 + i: outputs i - 1 .. i + 1 of this run, of which i + 1 begins and i - 1 is complete
                 const int lo = max(i - 1, 0), cnt = min(i + 1, n - 1) - lo + 1;
-                ok = mbar_wait(pfull + slot, pphase, kPolls);
+                ok = mbar_wait(pfull + slot, pphase, a.fault.limit<FAULT>(p));
                 if (i + 1 < n) {
                     ok = ok && mbar_wait(tempty + fresh, acc_phase, kPolls);
                     if (++fresh == a.nacc) {
@@ -568,6 +582,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
         const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
         const int xx = m % a.pitch, yy = m / a.pitch;
         int acc = 0, turn = 0, col = u0 / a.D, z = u0 - col * a.D;
+        int last = 2;  // the plane that completes the output
         uint32_t acc_phase = 0;
         bool ok = true;
         // every accumulator starts from zero (an instruction covers one that begins and two that go on)
@@ -584,7 +599,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
         }
         for (int u = u0; u < u1 && ok; u++) {
             if (turn == grp) {
-                ok = __all_sync(0xffffffffu, mbar_wait(tfull + acc, acc_phase, kPolls));
+                ok = __all_sync(0xffffffffu, mbar_wait(tfull + acc, acc_phase, a.fault.limit<FAULT>(last)));
                 tc_fence_after();
                 const int y = col * a.by + yy;
                 const bool valid = ok && yy < a.by && xx < a.W && y < a.H;
@@ -601,9 +616,11 @@ __global__ void __launch_bounds__(kRingThreads, 1)
                 }
             }
             turn ^= 1;
+            last++;
             if (++z == a.D) {
                 z = 0;
                 col++;
+                last += 2;
             }
             if (++acc == a.nacc) {
                 acc = 0;
@@ -653,6 +670,7 @@ struct WgradArgs {
     int kb_per_cta;
     int nstage;
     uint32_t tmem_cols;
+    CopyFault fault;
 };
 
 // MN-major descriptor: atoms of 8 rows x `row_bytes`, `lbo` bytes apart along M/N, 8-row groups
@@ -756,7 +774,7 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_tc_kernel(const __grid_cons
         int tx = kb0 % a.tx, ty = (kb0 / a.tx) % a.ty, tz = kb0 / (a.tx * a.ty);
         int s = 0, st = 0;
         uint32_t phase = 1;  // a fresh empty barrier's preceding phase counts as complete
-        for (; s < nkb; s++) {
+        for (; s < nkb && !a.fault.out(s); s++) {
             if (!__all_sync(0xffffffffu, mbar_wait(empty + st, phase, kPolls))) {
                 if (lane == 0) counts[2] = 1;
                 break;
@@ -791,7 +809,7 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_tc_kernel(const __grid_cons
         int s = 0, st = 0;
         uint32_t phase = 0, off = 0;
         for (; s < nkb; s++) {
-            if (!__all_sync(0xffffffffu, mbar_wait(full + st, phase, kPolls))) {
+            if (!__all_sync(0xffffffffu, mbar_wait(full + st, phase, a.fault.limit(s)))) {
                 if (leader) counts[2] = 1;
                 break;
             }
@@ -881,6 +899,7 @@ struct WlineArgs {
     int nstage;
     uint32_t stage_bytes, x_bytes, bar_off;
     uint32_t tmem_cols;
+    CopyFault fault;
 };
 
 __device__ __forceinline__ void tma_load_5d(void* dst, const CUtensorMap* map, int c0, int c1, int c2, int c3, int c4,
@@ -938,7 +957,7 @@ struct WgradTurn {
     }
 };
 
-template <int KS>  // bx / 16
+template <int KS, bool FAULT>  // bx / 16; FAULT: with the test hook
 __global__ void __launch_bounds__(kThreads, 1) wgrad_line_kernel(const __grid_constant__ CUtensorMap tmx,
                                                                  const __grid_constant__ CUtensorMap tmd,
                                                                  WlineArgs a) {
@@ -988,7 +1007,7 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_line_kernel(const __grid_co
             int tx = kb0 % a.tx, ty = (kb0 / a.tx) % a.ty, z = kb0 / (a.tx * a.ty);
             int s = 0, st = 0;
             uint32_t phase = 1;  // a fresh empty barrier's preceding phase counts as complete
-            for (; s < nkb; s++) {
+            for (; s < nkb && !a.fault.out<FAULT>(s); s++) {
                 if (!mbar_wait(empty + st, phase, kPolls)) {
                     counts[2] = 1;
                     break;
@@ -1025,7 +1044,7 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_line_kernel(const __grid_co
         uint32_t phase = 0, off = 0;
         WgradTurn w;
         for (; s < nkb; s++) {
-            bool ok = mbar_wait(full + st, phase, kPolls);
+            bool ok = mbar_wait(full + st, phase, a.fault.limit<FAULT>(s));
             if (w.i == 0 && s > 0) ok = ok && mbar_wait(drained, (w.segment - 1) & 1, kPolls);
             if (!__all_sync(0xffffffffu, ok)) {
                 if (leader) counts[2] = 1;
@@ -1268,11 +1287,15 @@ static cudaError_t launch_ring(RingGeom& g, const void* x, int ldx, const void* 
     if (kmajor_map(&mx, 4, x, xd, xs, xb) != CUDA_SUCCESS || kmajor_map(&mw, 3, w, wd, ws, wb) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     const int np = a.cin / g.ck;
-    const auto kernel = g.ck == 32 ? conv3_ring_kernel<32, 1>
-                        : np == 1  ? conv3_ring_kernel<16, 1>
-                        : np == 2  ? conv3_ring_kernel<16, 2>
-                        : np == 3  ? conv3_ring_kernel<16, 3>
-                                   : conv3_ring_kernel<16, 4>;
+    const auto pick = [&](auto fault) {
+        constexpr bool F = decltype(fault)::value;
+        return g.ck == 32 ? conv3_ring_kernel<32, 1, F>
+               : np == 1  ? conv3_ring_kernel<16, 1, F>
+               : np == 2  ? conv3_ring_kernel<16, 2, F>
+               : np == 3  ? conv3_ring_kernel<16, 3, F>
+                          : conv3_ring_kernel<16, 4, F>;
+    };
+    const auto kernel = a.fault.stop_after < 0 ? pick(std::false_type()) : pick(std::true_type());
     cudaError_t e = raise_smem(kernel, kRingSmemCap, g.smem);
     if (e != cudaSuccess) return e;
     return launch(kernel, dim3((unsigned)g.ctas, (unsigned)g.groups), kRingThreads, g.smem, st, mx, mw, a);
@@ -1286,12 +1309,13 @@ cudaError_t conv3_tc(const void* x, int ldx, int cin, const void* w, int cout, v
     EncodeTiled enc = encoder();
     if (!enc) return cudaErrorNotSupported;
     RingGeom ring = ring_geom(cin, cout, D, H, W);
-    if (ring.ctas > 0 && g_stop_after < 0) {
+    if (ring.ctas > 0) {
         ring.a.y = reinterpret_cast<__nv_bfloat16*>(y);
         ring.a.ldy = ldy;
         ring.a.relu = relu;
         ring.a.mask = reinterpret_cast<const __nv_bfloat16*>(mask);
         ring.a.ldm = ldm;
+        ring.a.fault = {g_stop_after, g_polls};
         return launch_ring(ring, x, ldx, w, cout, st);
     }
     // channels per operand row: one row where cin fits in it (16, 32), else pieces of 64, the last one
@@ -1322,8 +1346,7 @@ cudaError_t conv3_tc(const void* x, int ldx, int cin, const void* w, int cout, v
     a.ldm = ldm;
     while (a.bn > 16 && tiles * (cout / a.bn) < 152 && cout % (a.bn / 2) == 0 && (a.bn / 2) % 16 == 0) a.bn /= 2;
     a.tmem_cols = a.bn <= 32 ? 32 : a.bn <= 64 ? 64 : 128;
-    a.stop_after = g_stop_after;
-    a.polls = g_polls;
+    a.fault = {g_stop_after, g_polls};
     alignas(64) CUtensorMap mx, mw;
     const cuuint64_t xd[4] = {(cuuint64_t)cin, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)D};
     const cuuint64_t xs[3] = {(cuuint64_t)ldx * 2, (cuuint64_t)ldx * 2 * W, (cuuint64_t)ldx * 2 * W * H};
@@ -1530,8 +1553,15 @@ static cudaError_t wgrad_line(EncodeTiled enc, const WlineGeom& g, const void* x
     a.x_bytes = g.x_bytes;
     a.bar_off = g.bar_off;
     a.tmem_cols = g.tmem_cols;
-    const auto kernel = g.bx == 64 ? wgrad_line_kernel<4> : g.bx == 48 ? wgrad_line_kernel<3>
-                        : g.bx == 32 ? wgrad_line_kernel<2> : wgrad_line_kernel<1>;
+    a.fault = {g_stop_after, g_polls};
+    const auto pick = [&](auto fault) {
+        constexpr bool F = decltype(fault)::value;
+        return g.bx == 64   ? wgrad_line_kernel<4, F>
+               : g.bx == 48 ? wgrad_line_kernel<3, F>
+               : g.bx == 32 ? wgrad_line_kernel<2, F>
+                            : wgrad_line_kernel<1, F>;
+    };
+    const auto kernel = a.fault.stop_after < 0 ? pick(std::false_type()) : pick(std::true_type());
     cudaError_t e = raise_smem(kernel, kSmemCap, g.smem);
     if (e != cudaSuccess) return e;
     e = launch(kernel, dim3((unsigned)g.mgroups, (unsigned)g.nchunk), kThreads, g.smem, st, mx, md, a);
@@ -1594,6 +1624,7 @@ cudaError_t wgrad_tc(const void* x, int ldx, int cin, const void* dy, int ldy, i
     a.kb_per_cta = g.kb_per_cta;
     a.nstage = g.nstage;
     a.tmem_cols = g.tmem_cols;
+    a.fault = {g_stop_after, g_polls};
     cudaError_t e = raise_smem(wgrad_tc_kernel, kSmemCap, g.smem);
     if (e != cudaSuccess) return e;
     e = launch(wgrad_tc_kernel, dim3((unsigned)(g.mgroups * g.ngroups), (unsigned)g.nchunk), kThreads, g.smem, st, mx,
@@ -1602,8 +1633,8 @@ cudaError_t wgrad_tc(const void* x, int ldx, int cin, const void* dy, int ldy, i
     return wgrad_sum(a.partial, g.nchunk, g.mtiles, cin, cout, g.bn, g.wa, 0, dw, st);
 }
 
-// test hook: later convolutions issue only their first stop_after stages (< 0: normal operation) and
-// give up waiting after `polls` polls (<= 0: the default)
+// test hook: later convolutions and weight gradients issue only their first stop_after stages or planes (< 0: normal
+// operation) and give up waiting for the others after `polls` polls (<= 0: the default)
 void unet_set_copy_fault(int stop_after, int polls) {
     g_stop_after = stop_after;
     g_polls = polls > 0 ? polls : kPolls;
