@@ -166,7 +166,7 @@ cudaError_t run_sample_adjoint(const Geom& g, const Workspace& w, int kind, int 
 
 // Solver workspace, allocated by the first pat_tv_prox / pat_bregman_solve call on a grid.
 struct SolverWs {
-    size_t n_img = 0, n_dat = 0;  // per-call sizes the buffers were made for
+    size_t n_img = 0, n_dat = 0;  // sizes the image and data buffers were made for; 0: not all of them are there
     float *x = nullptr, *xp = nullptr, *y = nullptr, *z = nullptr, *grad = nullptr;  // image, B*N
     float *qbar = nullptr, *qbar2 = nullptr, *xi = nullptr, *xi2 = nullptr;         // prox: N, N, 3N, 3N
     float* q2 = nullptr;                                                            // prox: N

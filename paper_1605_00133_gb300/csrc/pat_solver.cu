@@ -570,39 +570,54 @@ static pat_status reduce(Ctx& c, const RedArgs* r, int n, double* out) {
     return PAT_OK;
 }
 
+// A buffer of the workspace, unless it is there: a call that ran out of memory leaves some of them, and the next one
+// goes on from there.
+template <class T>
+static pat_status ensure(pat_grid* G, T** p, size_t count, const char* what) {
+    if (*p) return PAT_OK;
+    void* q = nullptr;
+    const pat_status st = grid_alloc(G, &q, count * sizeof(T), what);
+    if (st == PAT_OK) *p = (T*)q;
+    return st;
+}
+
 static pat_status ensure_ws(pat_grid* G, bool solver) {
     SolverWs& w = G->sw;
     const size_t N = (size_t)G->g.B * G->g.nreal;
     const size_t D = (size_t)G->g.B * G->g.T * (size_t)G->m;
     pat_status st = PAT_OK;
-    if (!w.qbar) {
-        st = grid_alloc(G, (void**)&w.qbar, N * sizeof(float), "prox qbar");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.qbar2, N * sizeof(float), "prox qbar");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.xi, 3 * N * sizeof(float), "prox dual");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.xi2, 3 * N * sizeof(float), "prox dual");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.z, N * sizeof(float), "prox input copy");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.q2, N * sizeof(float), "prox iterate");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.partial, kRedMost * kRedBlocks * sizeof(double), "reduction");
-        if (st == PAT_OK) {
+    if (!w.n_img) {
+        st = ensure(G, &w.qbar, N, "prox qbar");
+        if (st == PAT_OK) st = ensure(G, &w.qbar2, N, "prox qbar");
+        if (st == PAT_OK) st = ensure(G, &w.xi, 3 * N, "prox dual");
+        if (st == PAT_OK) st = ensure(G, &w.xi2, 3 * N, "prox dual");
+        if (st == PAT_OK) st = ensure(G, &w.z, N, "prox input copy");
+        if (st == PAT_OK) st = ensure(G, &w.q2, N, "prox iterate");
+        if (st == PAT_OK) st = ensure(G, &w.partial, kRedMost * kRedBlocks, "reduction");
+        if (st == PAT_OK && !w.host) {
             cudaError_t e = cudaMallocHost((void**)&w.host, 4 * sizeof(double));
-            if (e != cudaSuccess) return set_cuda_error(e, "cudaMallocHost(reduction)");
+            if (e != cudaSuccess) {
+                w.host = nullptr;
+                return set_cuda_error(e, "cudaMallocHost(reduction)");
+            }
         }
         if (st != PAT_OK) return st;
         w.n_img = N;
     }
-    if (solver && !w.x) {
-        st = grid_alloc(G, (void**)&w.x, N * sizeof(float), "solver x");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.xp, N * sizeof(float), "solver x_prev");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.y, N * sizeof(float), "solver y");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.grad, N * sizeof(float), "solver gradient");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.ax, std::max<size_t>(D, 1) * sizeof(float), "solver Ax");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.axp, std::max<size_t>(D, 1) * sizeof(float), "solver Ax_prev");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.ay, std::max<size_t>(D, 1) * sizeof(float), "solver Ay");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.r, std::max<size_t>(D, 1) * sizeof(float), "solver residual");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.gdat, std::max<size_t>(D, 1) * sizeof(double), "solver data");
-        if (st == PAT_OK) st = grid_alloc(G, (void**)&w.bdat, std::max<size_t>(D, 1) * sizeof(double), "solver Bregman");
+    if (solver && !w.n_dat) {
+        const size_t data = std::max<size_t>(D, 1);
+        st = ensure(G, &w.x, N, "solver x");
+        if (st == PAT_OK) st = ensure(G, &w.xp, N, "solver x_prev");
+        if (st == PAT_OK) st = ensure(G, &w.y, N, "solver y");
+        if (st == PAT_OK) st = ensure(G, &w.grad, N, "solver gradient");
+        if (st == PAT_OK) st = ensure(G, &w.ax, data, "solver Ax");
+        if (st == PAT_OK) st = ensure(G, &w.axp, data, "solver Ax_prev");
+        if (st == PAT_OK) st = ensure(G, &w.ay, data, "solver Ay");
+        if (st == PAT_OK) st = ensure(G, &w.r, data, "solver residual");
+        if (st == PAT_OK) st = ensure(G, &w.gdat, data, "solver data");
+        if (st == PAT_OK) st = ensure(G, &w.bdat, data, "solver Bregman");
         if (st != PAT_OK) return st;
-        w.n_dat = D;
+        w.n_dat = data;
     }
     return PAT_OK;
 }
