@@ -637,7 +637,9 @@ static void tv2_plan(const TvDims& d, int B, TvStep2* a, dim3* grid, int* thread
     const int gx = a->split ? (d.nx + kTv2Cols - 1) / kTv2Cols : 1, gy = (d.ny + H - 1) / H;
     const long long tiles = (long long)gx * gy * B;
     *threads = (H + 3) * a->ntx;
-    const int resident = 152 * std::max(1, kTv2Threads / *threads);
+    // CTAs resident: 14 warps an SM (of 139 registers a thread).  Counted as 384 threads, which narrow tiles do not reach,
+    // 50 iterations of 128x256x16 took 309 us, now 271
+    const int resident = 152 * std::max(1, 14 / ((*threads + 31) / 32));
     long long best = 0;
     for (int run = 1; run <= d.nz; run++) {
         const int n = (d.nz + run - 1) / run;
@@ -709,17 +711,7 @@ static pat_status tv_prox_run(Ctx& c, const float* p, float* q, double alpha, in
                 next(&a.sigma[k], &a.tau[k], &a.theta[k]);
                 a.inv[k] = 1.f / (1.f + a.tau[k]);
             }
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = grid;
-            cfg.blockDim = dim3(threads);
-            cfg.dynamicSmemBytes = smem;
-            cfg.stream = c.st;
-            cudaLaunchAttribute at;
-            at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            at.val.programmaticStreamSerializationAllowed = 1;
-            cfg.attrs = &at;
-            cfg.numAttrs = 1;
-            PAT_CUDA(cudaLaunchKernelEx(&cfg, tv_step2_kernel, a), "prox launch");
+            PAT_CUDA(launch_pdl(tv_step2_kernel, grid, threads, smem, c.st, a), "prox launch");
         }
     }
     // what is left (an odd iteration; all of them for unaligned images) one at a time, in place on q

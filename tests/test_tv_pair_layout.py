@@ -26,7 +26,7 @@ def plan(nz, ny, nx, B):
         H = 8
     gx, gy = (nx + COLS - 1) // COLS if split else 1, (ny + H - 1) // H
     threads = (H + 3) * ntx
-    resident = 152 * max(1, THREADS // threads)
+    resident = 152 * max(1, 14 // -(-threads // 32))
     best = None
     for run in range(1, nz + 1):
         n = (nz + run - 1) // run
