@@ -895,7 +895,7 @@ struct WlineArgs {
     int bx, R, lines;   // voxels per line, lines of a block, lines of X fetched for it
     int tx, ty, nkb;    // blocks along x and y, in all
     int kb_per_cta;
-    int nset, seg;      // accumulators taking K blocks in turn; K blocks after which they are added up
+    int nset, seg;      // accumulators (1 or 2) taking K blocks in turn; K blocks after which they are added up
     int nstage;
     uint32_t stage_bytes, x_bytes, bar_off;
     uint32_t tmem_cols;
@@ -944,18 +944,6 @@ __device__ __forceinline__ void wgrad_store_sum(uint32_t taddr, int nset, int se
         }
     }
 }
-
-// Where the MMA issuer is: the segment, its K block, and the accumulator of that.
-struct WgradTurn {
-    int i = 0, set = 0, segment = 0;
-    __device__ __forceinline__ void next(int nset, int seg) {
-        if (++set == nset) set = 0;
-        if (++i == seg) {
-            i = set = 0;
-            segment++;
-        }
-    }
-};
 
 template <int KS, bool FAULT>  // bx / 16; FAULT: with the test hook
 __global__ void __launch_bounds__(kThreads, 1) wgrad_line_kernel(const __grid_constant__ CUtensorMap tmx,
@@ -1040,49 +1028,45 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_line_kernel(const __grid_co
         const uint64_t bd = mnmajor_desc(smem_addr(smem) + a.x_bytes, rb, rb);
         const uint32_t ahi = hi32(ad), bhi = hi32(bd), stage16 = a.stage_bytes >> 4;
         const uint32_t tile16 = (kBM / a.wa) * unit >> 4, aline16 = 3 * a.cb * unit >> 4, bline16 = (a.bx + 2) * rb >> 4;
-        int s = 0, st = 0;
+        int s = 0, st = 0, segment = 0;
         uint32_t phase = 0, off = 0;
-        WgradTurn w;
-        for (; s < nkb; s++) {
-            bool ok = mbar_wait(full + st, phase, a.fault.limit<FAULT>(s));
-            if (w.i == 0 && s > 0) ok = ok && mbar_wait(drained, (w.segment - 1) & 1, kPolls);
-            if (!__all_sync(0xffffffffu, ok)) {
-                if (leader) counts[2] = 1;
-                break;
-            }
-            tc_fence_after();
-            uint32_t al = lo32(ad) + off, td = tmem + w.set * set_cols;
-            const uint32_t bl = lo32(bd) + off;
-            for (int t = 0; t < mt; t++, al += tile16, td += ncols) {
-                uint32_t alo = al, blo = bl, on = w.i >= a.nset ? 1u : 0u;
-                for (int r = 0; r < a.R; r++, alo += aline16, blo += bline16) {
-                    // 16 voxel rows: the starts move by 16 rows of each operand
+        for (bool ok = true; ok && s < nkb; segment++) {
+            // accumulators handed back by the epilogue of the segment before
+            if (segment > 0) ok = __all_sync(0xffffffffu, mbar_wait(drained, (segment - 1) & 1, kPolls));
+            const int end = min(nkb, s + a.seg);
+            for (int i = 0; ok && s < end; i++, s++) {
+                ok = __all_sync(0xffffffffu, mbar_wait(full + st, phase, a.fault.limit<FAULT>(s)));
+                if (!ok) break;
+                tc_fence_after();
+                uint32_t al = lo32(ad) + off, td = tmem + ((i & (a.nset - 1)) ? set_cols : 0);
+                const uint32_t bl = lo32(bd) + off;
+                for (int t = 0; t < mt; t++, al += tile16, td += ncols) {
+                    uint32_t alo = al, blo = bl, on = i >= a.nset ? 1u : 0u;
+                    for (int r = 0; r < a.R; r++, alo += aline16, blo += bline16) {
+                        // 16 voxel rows: the starts move by 16 rows of each operand
 #pragma unroll
-                    for (int k = 0; k < KS; k++)
-                        tc_mma_if(leader, td, alo + k * ra, ahi, blo + k * rb, bhi, idesc, k ? 1u : on);
-                    on = 1u;
+                        for (int k = 0; k < KS; k++)
+                            tc_mma_if(leader, td, alo + k * ra, ahi, blo + k * rb, bhi, idesc, k ? 1u : on);
+                        on = 1u;
+                    }
+                }
+                if (leader) tc_commit(empty + st);
+                __syncwarp();
+                off += stage16;
+                if (++st == nstage) {
+                    st = 0;
+                    phase ^= 1;
+                    off = 0;
                 }
             }
             if (leader) {
-                tc_commit(empty + st);
-                if (w.i + 1 == a.seg && s + 1 < nkb) tc_commit(done);
+                if (!ok) counts[2] = 1;
+                counts[1] = s;
+                tc_commit(done);
             }
-            __syncwarp();
-            w.next(a.nset, a.seg);
-            off += stage16;
-            if (++st == nstage) {
-                st = 0;
-                phase ^= 1;
-                off = 0;
-            }
-        }
-        if (leader) {
-            counts[1] = s;
-            tc_commit(done);
         }
         __syncwarp();
-        // every MMA has finished before the tensor memory is freed (a loop that ended at nkb is in its last segment)
-        mbar_wait(done, (s == nkb ? (nkb - 1) / a.seg : w.segment) & 1, kPolls);
+        mbar_wait(done, (segment - 1) & 1, kPolls);  // every MMA has finished before the tensor memory is freed
     } else if (warp >= 2) {
         // epilogue: adds up the accumulators of each segment once it is done, and hands them back
         const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
