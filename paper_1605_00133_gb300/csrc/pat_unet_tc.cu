@@ -1302,9 +1302,6 @@ cudaError_t conv3_tc(const void* x, int ldx, int cin, const void* w, int cout, v
         ring.a.fault = {g_stop_after, g_polls};
         return launch_ring(ring, x, ldx, w, cout, st);
     }
-    // channels per operand row: one row where cin fits in it (16, 32), else pieces of 64, the last one
-    // zero-filled past cin
-    const int ck = cin == 16 ? 16 : cin == 32 ? 32 : 64;
     ConvTcArgs a = {};
     a.y = reinterpret_cast<__nv_bfloat16*>(y);
     a.ldy = ldy;
@@ -1333,6 +1330,12 @@ cudaError_t conv3_tc(const void* x, int ldx, int cin, const void* w, int cout, v
     while (a.bn > 16 && 2 * tiles * (cout / a.bn) <= 152 && cout % (a.bn / 2) == 0 && (a.bn / 2) % 16 == 0) a.bn /= 2;
     a.tmem_cols = a.bn <= 32 ? 32 : a.bn <= 64 ? 64 : 128;
     a.fault = {g_stop_after, g_polls};
+    // channels per operand row: one row where cin fits in it (16, 32), else pieces of 64, the last one zero-filled past
+    // cin.  But 96 and 160 channels in whole pieces of 32, of which more CTAs fit an SM, where more than one has to:
+    // 96 -> 32 at 32x64x64 voxels 54.4 us, in pieces of 64 69.2, 160 -> 32 86.6 and 97.5.  With a CTA an SM at most
+    // the fewer steps of 64 win: 96 -> 32 at 16x32x32 12.7 us, in pieces of 32 16.1; with 224 channels and more too
+    // (32x64x64, 128 outputs: 188 and 192)
+    const int ck = cin == 16 ? 16 : cin == 32 || ((cin == 96 || cin == 160) && tiles * (cout / a.bn) > 152) ? 32 : 64;
     alignas(64) CUtensorMap mx, mw;
     const cuuint64_t xd[4] = {(cuuint64_t)cin, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)D};
     const cuuint64_t xs[3] = {(cuuint64_t)ldx * 2, (cuuint64_t)ldx * 2 * W, (cuuint64_t)ldx * 2 * W * H};
