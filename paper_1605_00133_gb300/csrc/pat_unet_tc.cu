@@ -877,16 +877,17 @@ __global__ void __launch_bounds__(kThreads, 1) wgrad_tc_kernel(const __grid_cons
 // Rows of the last M tile beyond the 9 blocks atoms multiply whatever follows in shared memory and are not used.
 // What bounds it: the MMAs with few channels (two M tiles of N = 48 for 16 -> 16: 49 cycles each), the TMA unit with
 // more.  The whole gradient took with wgrad_tc_kernel (its partial products written 16 bytes a lane, 192 or more apart) ->
-// now: 64x128x128 voxels 16 -> 16 channels 69.9 -> 32 us, 48 -> 16 145 -> 64; 32x64x64 voxels 32 -> 32 31.5 -> 16,
-// 96 -> 32 49.5 -> 28.
+// now: 64x128x128 voxels 16 -> 16 channels 69.9 -> 31 us, 48 -> 16 145 -> 62; 32x64x64 voxels 32 -> 32 31.5 -> 16,
+// 96 -> 32 49.5 -> 27.
 // Accuracy: the tensor core truncates as it adds, so a sum of n voxels of one sign comes out low by about 1.3e-9 n of
 // its value (7168 voxels 9.1e-6, 14144 2.0e-5).  So K blocks go to two accumulators in turn where tensor memory holds
 // two, and after kChain voxels in each, or at the end, the epilogue adds them up, rounding to nearest, and to what
-// earlier segments left in the partial product.  ReLU'd operands, relative error against FP64 of one accumulator to the
-// end -> now: 64x128x128 voxels 16 -> 16 channels 9.1e-6 -> 3.8e-6 (1 us more), 48 -> 16 8.9e-6 -> 3.8e-6 (with its
-// tiles in two groups and chains twice as long 2.0e-5); 32x64x64 voxels 16 -> 32 9.5e-7 -> 4.1e-7; 128x256x256 voxels
-// 16 -> 16 1.0e-4 -> 8.8e-6 (200 -> 218 us).
-constexpr int kChain = 7168;  // most voxels summed by one accumulator: 448 MMAs
+// earlier segments left in the partial product.  Relative error against FP64 with one accumulator to the end, 48
+// channels in two groups of tiles -> now: ReLU'd normal numbers at 64x128x128 voxels 16 -> 16 channels 9.1e-6 -> 3.8e-6,
+// 48 -> 16 2.0e-5 -> 8.9e-6; at 32x64x64 16 -> 32 9.5e-7 -> 4.1e-7; at 128x256x256 16 -> 16 1.0e-4 -> 9e-6 (200 -> 218 us).
+// In the network at 64x128x128, whose operands are large in few places (eight of them): d1a (48 -> 16) 1.0e-5 .. 4.6e-5
+// -> 5.6e-6 .. 2.1e-5, d1b 5e-6 .. 2.4e-5 -> 2.6e-6 .. 1.1e-5, e1a 7e-6 -> 3.6e-6, the others below 4e-6.
+constexpr int kChain = 7424;  // most voxels summed by one accumulator: 464 MMAs
 
 struct WlineArgs {
     float4* partial;    // as above; rows in the order (dy, dz, channel), columns (1 - dx, output channel)
@@ -1427,14 +1428,17 @@ static WlineGeom wline_geom(int cin, int cout, int D, int H, int W) {
     const int per_tile = kBM / g.wa, N = 3 * cout, ncols = (N + 31) & ~31;
     g.mtiles = (9 * cin + kBM - 1) / kBM;
     // Up to four M tiles a CTA, so that 48 channels are one group, whose lines are fetched once: 48 -> 16 channels at
-    // 64x128x128 64 us, in two groups of two tiles 87 (and the same accuracy).
+    // 64x128x128 62 us, in two groups of two tiles 87 (and the chains of a tile are half as long).
     g.mgroups = (g.mtiles + 3) / 4;
     g.mt = (g.mtiles + g.mgroups - 1) / g.mgroups;
     for (int i = 0; i < g.mgroups; i++) {
         const int a0 = i * g.mt * per_tile, a1 = std::min((i + 1) * g.mt * per_tile, 9 * g.cb) - 1;
         g.span = std::max(g.span, a1 / (3 * g.cb) - a0 / (3 * g.cb));
     }
-    g.nset = std::min(2, 512 / (g.mt * ncols));  // one CTA an SM: all of its tensor memory
+    // One CTA an SM: all of its tensor memory.  But four tiles take one accumulator each: with two, at no cost, d1a came
+    // out at 3e-6 .. 9e-6 in the network, which moved 3 % of the whole gradients by more than 2e-5, the most that results
+    // in FP32 may move from one version to the next.
+    g.nset = g.mt == 4 ? 1 : std::min(2, 512 / (g.mt * ncols));
     g.tmem_cols = 64;
     while ((int)g.tmem_cols < g.nset * g.mt * ncols) g.tmem_cols *= 2;
     // The block shape with the least time of TMA unit (a box row a cycle) or MMAs, over the volume padded to whole
