@@ -591,9 +591,10 @@ __device__ __forceinline__ void line_pass(const LineArgs& a, int tile) {
     if (!PARTS && !late) pdl_wait();
     if (!PARTS && !(a.flags & (LF_TRIGGER_MID | LF_TRIGGER_END))) pdl_trigger();
     constexpr int XN = S::XN;
-    // The two halves (factor, inverse transform, state update, transform) as one loop body: half the code, so fewer
-    // waits for instructions (0.4 cycles of 8 per instruction before).  64x128x128, forward over 400 steps: 7.49 ->
-    // 7.33 ms at L = 128 only, 7.31 at 64 too; 64^3 in one launch a step (pat_step.cuh) 498 -> 451 us over 64 steps.
+    // The two halves (factor, inverse transform, state update, transform) as one loop body: half the code and 5 %
+    // fewer instructions (x pass of 64x128x128 4.31 -> 4.08 M warp instructions; a captured launch with cold caches
+    // waits for instructions as much as before).  Forward over 400 steps of it: 7.49 -> 7.33 ms at L = 128 only, 7.31
+    // at 64 too; 64^3 in one launch a step (pat_step.cuh) 498 -> 451 us over 64 steps.
     // Shorter lines gain nothing (32^3 293 -> 297 us), L = 256 lost.
     constexpr bool ROLLED = L == 64 || L == 128;
     static_assert(!ROLLED || (S::BULK && !S::PFO_ALIAS), "tiles of the rolled form");

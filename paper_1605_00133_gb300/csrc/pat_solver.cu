@@ -235,8 +235,9 @@ __global__ void __launch_bounds__(32 * kTvWarps) tv_step_kernel(TvStep a) {
 // of z planes and marches along z; a thread holds four consecutive x of one row.  At plane z it evaluates
 // the first iteration's dual and primal there and the second iteration's for plane z - 1, which needs the first
 // one's over-relaxed iterate at z.  What the second iteration reads of neighbouring tiles is evaluated
-// redundantly: duals of rows y0 - 2 .. y0 + H and y0 - 1 .. y0 + H - 1, primals one row less (at H = 8: 20
-// and 18 rows for 16), and three planes more than a run stores.  Neighbours along x and y come through
+// redundantly: all H + 3 rows y0 - 2 .. y0 + H in both iterations (of which the second needs two less, and the primals
+// one less), and three planes more than a run stores (the second dual two).  At 64x128x128 (H = 8, runs of 8) that is
+// 1.8 dual evaluations per voxel and iteration, at 128x256x256 1.68.  Neighbours along x and y come through
 // shared memory (two barriers per plane for both iterations), along z through registers; a plane's inputs
 // are fetched while the one before is computed.  Per voxel the operations are tv_step_kernel's, in the same
 // order, so the results are the same bit for bit.  20 iterations of 128x256x256 2193 -> 1101 us,
